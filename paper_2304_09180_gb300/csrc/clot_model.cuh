@@ -52,6 +52,29 @@ __device__ __forceinline__ float affinity(const RxnConst& k, float eta) {
 // on the species-step path; the surrogate's training pairs use double.
 // y and f hold at least the CLOT_NS species (the inhibitor extension's two
 // rows may follow; they are not touched here).
+//
+// Every rounding is spelled out (mul_ and fma_ below, never an expression the
+// compiler may contract one way or the other): the kernels that share this
+// code then give the same bits, also for concentrations among the subnormal
+// numbers, where another contraction shows.
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// The injury-face exchange: J, the rates of E0 and C0, and what S1, E1 gain.
+template <typename T>
+__device__ __forceinline__ void wall_rhs(const RxnConst& k, T s1, T e0, T c0, T& fs1, T& fe1, T& fe0, T& fc0) {
+  const T un = mul_((T)k.kC0m, c0);
+  const T s1w = fma_((T)k.Dd, s1, un) / fma_((T)k.kC0p, e0, (T)k.Dd);
+  const T J = fma_(mul_((T)k.kC0p, s1w), e0, -un);
+  const T cat0 = mul_((T)k.kC0cat, c0);
+  fs1 = fma_(-(T)k.aV, J, fs1);
+  fe1 = fma_((T)k.aV, cat0, fe1);
+  fe0 = fma_((T)k.kC0cat, c0, -J);
+  fc0 = fma_(-(T)k.kC0cat, c0, J);
+}
+
 template <bool WALL, typename T = float>
 __device__ __forceinline__ void rxn_rhs(const RxnConst& k, const T* y, T adhH, T A1, T coh, T e0, T c0, T* f,
                                         T& fe0, T& fc0) {
@@ -60,42 +83,35 @@ __device__ __forceinline__ void rxn_rhs(const RxnConst& k, const T* y, T adhH, T
   const T s1b = y[CLOT_S1B], s2b = y[CLOT_S2B], e1b = y[CLOT_E1B], e2b = y[CLOT_E2B];
   const T c1 = y[CLOT_C1], c2 = y[CLOT_C2];
 
-  const T adh = adhH * (k.Pmax - Pbse);
-  const T A = A1 + k.k_e2 * e2 / (k.e2_star + e2);
-  f[CLOT_PMU] = -adh * Pmu - A * Pmu;
-  f[CLOT_PMA] = -adh * Pma + A * Pmu - coh * Pma;
-  f[CLOT_PBA] = -adh * Pba + coh * Pma;
-  f[CLOT_PBSE] = adh * (Pmu + Pma + Pba);
+  const T adh = mul_(adhH, (T)k.Pmax - Pbse);
+  const T A = A1 + mul_((T)k.k_e2, e2) / ((T)k.e2_star + e2);
+  const T act = mul_(A, Pmu), ch = mul_(coh, Pma);
+  f[CLOT_PMU] = fma_(-adh, Pmu, -act);
+  f[CLOT_PMA] = fma_(-adh, Pma, act) - ch;
+  f[CLOT_PBA] = fma_(-adh, Pba, ch);
+  f[CLOT_PBSE] = mul_(adh, Pmu + Pma + Pba);
 
   const T sites = Pba + Pbse;
-  const T free1 = k.n1 * sites - (s1b + e1b + c1 + c2);
-  const T free2 = k.n2 * sites - (s2b + e2b + c1 + c2);
-  const T bS1 = k.kS1p * free1 * s1 - k.kS1m * s1b;  // net binding S1 -> S1b
-  const T bE1 = k.kE1p * free1 * e1 - k.kE1m * e1b;
-  const T bS2 = k.kS2p * free2 * s2 - k.kS2m * s2b;
-  const T bE2 = k.kE2p * free2 * e2 - k.kE2m * e2b;
-  const T a1 = k.kC1p * s2b * e1b - k.kC1m * c1;     // net association into C1
-  const T a2 = k.kC2p * s1b * e2b - k.kC2m * c2;     // net association into C2
-  const T cat1 = k.kC1cat * c1, cat2 = k.kC2cat * c2;
+  const T free1 = fma_((T)k.n1, sites, -(s1b + e1b + c1 + c2));
+  const T free2 = fma_((T)k.n2, sites, -(s2b + e2b + c1 + c2));
+  const T bS1 = fma_(mul_((T)k.kS1p, free1), s1, -mul_((T)k.kS1m, s1b));  // net binding S1 -> S1b
+  const T bE1 = fma_(mul_((T)k.kE1p, free1), e1, -mul_((T)k.kE1m, e1b));
+  const T bS2 = fma_(mul_((T)k.kS2p, free2), s2, -mul_((T)k.kS2m, s2b));
+  const T bE2 = fma_(mul_((T)k.kE2p, free2), e2, -mul_((T)k.kE2m, e2b));
+  const T a1 = fma_(mul_((T)k.kC1p, s2b), e1b, -mul_((T)k.kC1m, c1));     // net association into C1
+  const T a2 = fma_(mul_((T)k.kC2p, s1b), e2b, -mul_((T)k.kC2m, c2));     // net association into C2
+  const T q1 = (T)k.kC1cat, q2 = (T)k.kC2cat;
   f[CLOT_S1] = -bS1;
   f[CLOT_S2] = -bS2;
   f[CLOT_E1] = -bE1;
   f[CLOT_E2] = -bE2;
   f[CLOT_S1B] = bS1 - a2;
   f[CLOT_S2B] = bS2 - a1;
-  f[CLOT_E1B] = bE1 - a1 + cat1 + cat2;
-  f[CLOT_E2B] = bE2 - a2 + cat2 + cat1;
-  f[CLOT_C1] = a1 - cat1;
-  f[CLOT_C2] = a2 - cat2;
-  if (WALL) {
-    const T s1w = (k.Dd * s1 + k.kC0m * c0) / (k.Dd + k.kC0p * e0);
-    const T J = k.kC0p * s1w * e0 - k.kC0m * c0;
-    const T cat0 = k.kC0cat * c0;
-    f[CLOT_S1] -= k.aV * J;
-    f[CLOT_E1] += k.aV * cat0;
-    fe0 = cat0 - J;
-    fc0 = J - cat0;
-  }
+  f[CLOT_E1B] = fma_(q2, c2, fma_(q1, c1, bE1 - a1));
+  f[CLOT_E2B] = fma_(q1, c1, fma_(q2, c2, bE2 - a2));
+  f[CLOT_C1] = fma_(-q1, c1, a1);
+  f[CLOT_C2] = fma_(-q2, c2, a2);
+  if (WALL) wall_rhs(k, s1, e0, c0, f[CLOT_S1], f[CLOT_E1], fe0, fc0);
 }
 
 // rxn_rhs with the injury-wall exchange switched at run time (fe0, fc0 are
@@ -103,15 +119,7 @@ __device__ __forceinline__ void rxn_rhs(const RxnConst& k, const T* y, T adhH, T
 __device__ __forceinline__ void rxn_rhs_rt(const RxnConst& k, const float* y, float adhH, float A1, float coh,
                                            bool wall, float e0, float c0, float* f, float& fe0, float& fc0) {
   rxn_rhs<false>(k, y, adhH, A1, coh, e0, c0, f, fe0, fc0);
-  if (wall) {
-    const float s1w = (k.Dd * y[CLOT_S1] + k.kC0m * c0) / (k.Dd + k.kC0p * e0);
-    const float J = k.kC0p * s1w * e0 - k.kC0m * c0;
-    const float cat0 = k.kC0cat * c0;
-    f[CLOT_S1] -= k.aV * J;
-    f[CLOT_E1] += k.aV * cat0;
-    fe0 = cat0 - J;
-    fc0 = J - cat0;
-  }
+  if (wall) wall_rhs(k, y[CLOT_S1], e0, c0, f[CLOT_S1], f[CLOT_E1], fe0, fc0);
 }
 
 // Row indices of the inhibitor extension's species after the CLOT_NS cell
@@ -122,7 +130,7 @@ constexpr int CLOT_NX = CLOT_NS + 2, XINH = CLOT_NS, XE2I = CLOT_NS + 1;
 // I + E2 -> E2,inh at rate kI I E2): fluid-phase thrombin and I each lose
 // kI I E2, E2,inh gains it.
 __device__ __forceinline__ void inhibit_rhs(const RxnConst& k, const float* y, float* f) {
-  const float r = k.kI * y[XINH] * y[CLOT_E2];
+  const float r = mul_(mul_(k.kI, y[XINH]), y[CLOT_E2]);
   f[CLOT_E2] -= r;
   f[XINH] = -r;
   f[XE2I] = r;
@@ -165,32 +173,32 @@ __device__ __forceinline__ float rxn_rk4(const RxnConst& k, float (&y)[N], float
 #pragma unroll
     for (int q = 0; q < N; ++q) {
       acc[q] = f[q];
-      yt[q] = (q == CLOT_ADP) ? y[q] : (y[q] + D[q]) + h2 * f[q];
+      yt[q] = (q == CLOT_ADP) ? y[q] : fma_(h2, f[q], y[q] + D[q]);
     }
     ae0 = fe0; ac0 = fc0;
     // stage 2
-    rhs(yt, be0 + h2 * fe0, bc0 + h2 * fc0, f, fe0, fc0);
+    rhs(yt, fma_(h2, fe0, be0), fma_(h2, fc0, bc0), f, fe0, fc0);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      acc[q] += 2.0f * f[q];
-      yt[q] = (q == CLOT_ADP) ? y[q] : (y[q] + D[q]) + h2 * f[q];
+      acc[q] = fma_(2.0f, f[q], acc[q]);
+      yt[q] = (q == CLOT_ADP) ? y[q] : fma_(h2, f[q], y[q] + D[q]);
     }
-    ae0 += 2.0f * fe0; ac0 += 2.0f * fc0;
+    ae0 = fma_(2.0f, fe0, ae0); ac0 = fma_(2.0f, fc0, ac0);
     // stage 3
-    rhs(yt, be0 + h2 * fe0, bc0 + h2 * fc0, f, fe0, fc0);
+    rhs(yt, fma_(h2, fe0, be0), fma_(h2, fc0, bc0), f, fe0, fc0);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      acc[q] += 2.0f * f[q];
-      yt[q] = (q == CLOT_ADP) ? y[q] : (y[q] + D[q]) + h * f[q];
+      acc[q] = fma_(2.0f, f[q], acc[q]);
+      yt[q] = (q == CLOT_ADP) ? y[q] : fma_(h, f[q], y[q] + D[q]);
     }
-    ae0 += 2.0f * fe0; ac0 += 2.0f * fc0;
+    ae0 = fma_(2.0f, fe0, ae0); ac0 = fma_(2.0f, fc0, ac0);
     // stage 4
-    rhs(yt, be0 + h * fe0, bc0 + h * fc0, f, fe0, fc0);
+    rhs(yt, fma_(h, fe0, be0), fma_(h, fc0, bc0), f, fe0, fc0);
 #pragma unroll
     for (int q = 0; q < N; ++q)
-      if (q != CLOT_ADP) D[q] += h6 * (acc[q] + f[q]);
-    De0 += h6 * (ae0 + fe0);
-    Dc0 += h6 * (ac0 + fc0);
+      if (q != CLOT_ADP) D[q] = fma_(h6, acc[q] + f[q], D[q]);
+    De0 = fma_(h6, ae0 + fe0, De0);
+    Dc0 = fma_(h6, ac0 + fc0, Dc0);
   }
 #pragma unroll
   for (int q = 0; q < N; ++q)
@@ -258,9 +266,8 @@ __device__ __forceinline__ bool rxn_linear_rest(const RxnConst& k, float (&y)[N]
   const float q = -z * (1.0f + z * (0.5f + z * ((1.0f / 6.0f) + z * (1.0f / 24.0f))));  // 1 - R(z)
   float pmu = y[CLOT_PMU], pma = y[CLOT_PMA];
   for (int m = 0; m < M; ++m) {
-    const float d = pmu * q;
-    pma += d;
-    pmu -= d;
+    pma = fma_(pmu, q, pma);
+    pmu = fma_(-pmu, q, pmu);
   }
   y[CLOT_PMU] = pmu;
   y[CLOT_PMA] = pma;
