@@ -40,10 +40,13 @@ struct clot_mesh {
   float* wall_lo;      // [2][max(n_inj, 1)] low words of E0, C0 (CLOT_DEVIATION)
   float* cg;           // [9][ncell] eta solver r, p, q, p2 and the single-reduction CG's five more
   float* eta_ws;       // [2][ncell] eta buffers of the step-to-step prediction
-  unsigned* maxw;      // [4] two sets of (max |r|, max theta_B) of the prediction
+  unsigned* maxw;      // two sets of (max |r|, max theta_B, max |r| of each 32 x 8 tile column) of the prediction
+  int tiles, nmaxw;    // tile columns recorded, words of a set
+  int dct;             // the direct eta solver takes this mesh
+  float* dct_tab;      // its cosine tables: y, then z
   double* partials;
   double* dout;        // [8]
-  unsigned* bar;       // [8] grid barrier words, box bounds of the eta correction
+  unsigned* bar;       // [16] grid barrier words, box bounds of the eta correction
   int* status;         // [8] flags, last eta iterations, summed iterations, accepted predictions, box fixes, box fallbacks
   unsigned long long* scount;  // [4] surrogate fallback counters and list length
   // eta prediction carried from one clot_species_step call to the next
@@ -53,7 +56,7 @@ struct clot_mesh {
   double pred_t, pred_dt;  // time of the next step, its dt
   float* pred_guess;       // workspace buffer holding the predicted eta of that step
   int pred_sel;            // maxima set the last fused step wrote
-  int eta_grid;
+  int cg_grid, dct_grid;  // blocks of the iterative and of the direct eta solve
   int aux_blocks;
   const float* vfx[2];  // the last two validated (fluxes, dt) sets (double-buffered uploads)
   const float* vfy[2];
@@ -114,6 +117,7 @@ static void free_mesh(clot_mesh* m) {
   cudaFree(m->cg);
   cudaFree(m->eta_ws);
   cudaFree(m->maxw);
+  cudaFree(m->dct_tab);
   cudaFree(m->partials);
   cudaFree(m->dout);
   cudaFree(m->bar);
@@ -187,33 +191,50 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
   // 1024 x 256 channel one block per 2048 cells took 0.91 ms of eta per primed
   // step against 1.23 ms with one per 512 cells (and 1.10 with one per 8192).
   const long long need = (g.ncell + 4 * ETA_BLOCK - 1) / (4 * ETA_BLOCK);
-  m->eta_grid = (int)std::min<long long>(grid, std::max<long long>(need, 1));
+  m->cg_grid = (int)std::min<long long>(grid, std::max<long long>(need, 1));
+  // The direct solver replaces the iteration wherever its tables stay small:
+  // from zero on the 512 x 128 x 128 duct 0.27 ms against 3.4 ms (44 CG
+  // iterations), per primed step of the 1024 x 256 channel 0.043 against 0.62 ms
+  // (37 iterations), with a smaller error (2.8e-7 against 4.2e-7 of eta).
+  m->dct = dct_applies(g) ? 1 : 0;
+  const long long ntile = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+  m->tiles = ntile <= 4096 ? (int)ntile : 0;  // every block of the eta solve reads them
+  m->nmaxw = 2 + m->tiles;
+  const long long ty = m->dct ? dct_table_floats(g.ny) : 0, tz = m->dct && g.dim == 3 ? dct_table_floats(g.nz) : 0;
+  if (m->dct) {
+    m->dct_grid = dct_max_grid(g);
+    if (m->dct_grid < 1) { free_mesh(m); return fail(CLOT_ECUDA, "occupancy query failed"); }
+  }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
   m->aux_blocks = (int)std::min<long long>(std::max(sms, 1) * 8, std::max<long long>((g.ncell + 255) / 256, 1));
 
-  const size_t npart = (size_t)std::max(3 * m->eta_grid + 8, 8 * m->aux_blocks);
+  const size_t npart = (size_t)std::max(6 * std::max(m->cg_grid, m->dct_grid), 8 * m->aux_blocks);
   if (cudaMalloc(&m->scratch, sizeof(float) * CLOT_NS * g.pitch) != cudaSuccess ||
       cudaMalloc(&m->stage, sizeof(float) * CLOT_NS * g.pitch) != cudaSuccess ||
       cudaMalloc(&m->xws, sizeof(float) * 4 * g.pitch) != cudaSuccess ||
       cudaMalloc(&m->dev_in, sizeof(float) * 2 * (size_t)g.ny * g.nz) != cudaSuccess ||
       cudaMalloc(&m->wall_lo, sizeof(float) * 2 * (size_t)std::max(g.n_inj, 1)) != cudaSuccess ||
-      cudaMalloc(&m->cg, sizeof(float) * 9 * g.ncell) != cudaSuccess ||
+      cudaMalloc(&m->cg, sizeof(float) * (9 * g.ncell + 32)) != cudaSuccess ||
       cudaMalloc(&m->eta_ws, sizeof(float) * 2 * g.ncell) != cudaSuccess ||
-      cudaMalloc(&m->maxw, sizeof(unsigned) * 4) != cudaSuccess ||
+      cudaMalloc(&m->maxw, sizeof(unsigned) * 2 * m->nmaxw) != cudaSuccess ||
+      (m->dct && cudaMalloc(&m->dct_tab, sizeof(float) * (ty + tz)) != cudaSuccess) ||
       cudaMalloc(&m->partials, sizeof(double) * npart) != cudaSuccess ||
       cudaMalloc(&m->dout, sizeof(double) * 8) != cudaSuccess ||
-      cudaMalloc(&m->bar, sizeof(unsigned) * 8) != cudaSuccess ||
+      cudaMalloc(&m->bar, sizeof(unsigned) * 16) != cudaSuccess ||
       cudaMalloc(&m->status, sizeof(int) * 8) != cudaSuccess ||
       cudaMalloc(&m->scount, sizeof(unsigned long long) * 4) != cudaSuccess) {
     free_mesh(m);
     cudaGetLastError();
     return fail(CLOT_ENOMEM, "device allocation of the mesh workspace failed");
   }
-  if (cudaMemset(m->bar, 0, 8 * sizeof(unsigned)) != cudaSuccess ||
+  if (cudaMemset(m->bar, 0, 16 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(m->status, 0, 8 * sizeof(int)) != cudaSuccess ||
       cudaMemset(m->cg, 0, sizeof(float) * 4 * g.ncell) != cudaSuccess ||
-      cudaMemset(m->maxw, 0, sizeof(unsigned) * 4) != cudaSuccess) {
+      cudaMemset(m->maxw, 0, sizeof(unsigned) * 2 * m->nmaxw) != cudaSuccess ||
+      (m->dct && launch_dct_table(g.ny, m->dct_tab, 0) != cudaSuccess) ||
+      (tz && launch_dct_table(g.nz, m->dct_tab + ty, 0) != cudaSuccess) ||
+      (m->dct && cudaDeviceSynchronize() != cudaSuccess)) {
     free_mesh(m);
     return fail(CLOT_ECUDA, "workspace initialisation failed");
   }
@@ -415,7 +436,21 @@ static EtaArgs make_eta(clot_mesh* m, clot_fields* f, const clot_params* p, cons
   a.predicted = 0;
   a.maxw = nullptr;
   a.maxw_clear = nullptr;
+  a.eta_t = (float)p->eta_t;
+  a.tiles = m->tiles;
+  if (m->dct) {  // the eight vectors after r hold the two work fields (each at most 4 ncell: nx = 1)
+    a.dct_y = m->dct_tab;
+    a.dct_z = m->dct_tab + dct_table_floats(m->g.ny);
+    const long long n4 = (m->g.ncell + 3) / 4 * 4;
+    a.dct_a = m->cg + n4;
+    a.dct_b = m->cg + 5 * n4;
+  }
   return a;
+}
+
+static cudaError_t launch_eta(const clot_mesh* m, const EtaArgs& e, cudaStream_t s) {
+  // the direct solver divides by the x coupling; a run that couples no cells (L_eta = 0) iterates
+  return m->dct && e.cx > 0.0f ? launch_eta_dct(e, m->dct_grid, s) : launch_eta_solve(e, m->cg_grid, s);
 }
 
 // Read the device status word (synchronous) and clear its flags: the timeout
@@ -568,7 +603,7 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
     have_pred = true;
     sel0 = m->pred_sel ^ 1;
   } else if (predict) {
-    CUDA_OK(cudaMemsetAsync(m->maxw, 0, 4 * sizeof(unsigned), s));
+    CUDA_OK(cudaMemsetAsync(m->maxw, 0, 2 * m->nmaxw * sizeof(unsigned), s));
   }
   // Deviation form for the length of the call: the S1, S2 rows and their
   // inlet values shifted by the references (the rates add them back), the
@@ -603,10 +638,10 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       e.inner = 1.0f;  // no over-solve: measured fastest (CG iterations and accepted predictions)
       if (have_pred) {
         e.predicted = 1;
-        e.maxw = m->maxw + 2 * (sel ^ 1);      // written by the previous fused step
-        e.maxw_clear = m->maxw + 2 * sel;      // used by this step's fused kernel
+        e.maxw = m->maxw + m->nmaxw * (sel ^ 1);      // written by the previous fused step
+        e.maxw_clear = m->maxw + m->nmaxw * sel;      // used by this step's fused kernel
       }
-      CUDA_OK(traced(m, K_ETA, s, [&] { return launch_eta_solve(e, m->eta_grid, s); }));
+      CUDA_OK(traced(m, K_ETA, s, [&] { return launch_eta(m, e, s); }));
     }
     if (!(p->flags & CLOT_NO_SIGMA)) {
       SigmaArgs sa = make_sigma(m, f, p);
@@ -705,7 +740,8 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       A.eta_prev = eprev;
       A.eta_next = enext;
       A.eta_res = m->cg;
-      A.eta_max = m->maxw + 2 * sel;
+      A.eta_max = m->maxw + m->nmaxw * sel;
+      A.eta_tiles = m->tiles;
     }
     if (run_k1) {
       CUDA_OK(traced(m, K_STEP, s, [&] { return launch_species_step_plane(A, s); }));
@@ -843,7 +879,7 @@ extern "C" int clot_eta_solve(clot_mesh* m, clot_fields* f, const clot_params* p
   if ((rc = check_device(m)) || (rc = check_fields(m, f)) || (rc = check_params(m, p))) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   EtaArgs e = make_eta(m, f, p, f->c);
-  CUDA_OK(traced(m, K_ETA, s, [&] { return launch_eta_solve(e, m->eta_grid, s); }));
+  CUDA_OK(traced(m, K_ETA, s, [&] { return launch_eta(m, e, s); }));
   if (iters) return read_status(m, s, iters);
   return CLOT_OK;
 }

@@ -85,9 +85,10 @@ struct StepArgs {
   const float* __restrict__ eta_prev;
   float* eta_next;
   float* eta_res;
-  unsigned* eta_max;           // [2]: max |r|, max theta_B (float bit patterns, atomicMax)
+  unsigned* eta_max;           // max |r|, max theta_B (float bit patterns, atomicMax), then max |r| of each
+                               // 32 x 8 tile column if eta_tiles
   float ecx, ecy, ecz;         // (L_eta^2 / 4) / h_a^2
-  int predict;
+  int predict, eta_tiles;
   int* status;                 // device status word: ST_TIMEOUT when a bounded wait gives up (may be null)
   StepConst K;
 };
@@ -147,8 +148,9 @@ struct EtaArgs {
   float* p2;                    // second search-direction buffer (p_old / p_new alternate)
   float* cg5;                   // [5][ncell] second r, two s, two w buffers of the single-reduction CG
                                 // (null: the two-reduction CG)
-  double* partials;             // [3][gridDim] + 6 reduced scalars
-  unsigned* bar;                // [8] arrive counter, generation, box bounds of the predicted-eta fix
+  double* partials;             // [2][3][gridDim]
+  unsigned* bar;                // [10] arrivals, -, box bounds of the predicted-eta fix (6), departures,
+                                // max theta_B; zero at launch, and again when the launch ends
   int* status;                  // [0] flags, [1] iterations, [2] summed iterations, [3] accepted predictions,
                                 // [4] predictions corrected on a box, [5] box corrections that fell back
   Geom g;
@@ -160,8 +162,17 @@ struct EtaArgs {
   int maxit;
   int predicted;                // r and eta hold a predicted guess and its residual
   unsigned long long wait_ns;   // bound of each grid-barrier wait (globaltimer ns)
-  const unsigned* maxw;         // [2] max |r|, max theta_B of the prediction
-  unsigned* maxw_clear;         // [2] the other maxima set, zeroed for the next step
+  const unsigned* maxw;         // max |r|, max theta_B of the prediction, then (tiles > 0)
+                                // max |r| of each 32 x 8 tile column
+  unsigned* maxw_clear;         // the other maxima set, zeroed for the next step
+  // direct solver (clot_eta_dct.cu): cosine tables of the y and z axes and two
+  // work fields of ny nz (nx rounded up to 4) floats
+  float eta_t;                  // binding threshold of g(eta): the direct solver is for max theta_B above it
+  int tiles;                    // 32 x 8 tile columns whose max |r| follows maxw[0..1] (0: not recorded)
+  const float* dct_y;
+  const float* dct_z;
+  float* dct_a;
+  float* dct_b;
 };
 // The box correction of a predicted eta (App. A Eq. eta; used by the
 // single-mesh solver and the ensemble's block-per-channel solver): an
@@ -191,6 +202,17 @@ __device__ __forceinline__ int box_margin(float c, float rmax, float stop) {
 constexpr int ETA_BLOCK = 512;
 cudaError_t launch_eta_solve(const EtaArgs& a, int grid, cudaStream_t s);
 int eta_max_grid(int* grid_out);
+
+// Direct solver (clot_eta_dct.cu) for meshes of at most DCT_MAX_NX x DCT_MAX_N
+// (x DCT_MAX_N) cells: its dense transforms cost ny + nz multiply-adds a cell,
+// and a warp holds a whole x line in registers.
+constexpr int DCT_THREADS = 128, DCT_MAX_NX = 1024, DCT_MAX_N = 512;
+__host__ __device__ __forceinline__ int dct_half(int n) { return ((n + 1) / 2 + 63) / 64 * 64; }
+bool dct_applies(const Geom& g);
+int dct_max_grid(const Geom& g);
+long long dct_table_floats(int n);
+cudaError_t launch_dct_table(int n, float* out, cudaStream_t s);
+cudaError_t launch_eta_dct(const EtaArgs& a, int grid, cudaStream_t s);
 
 struct SigmaArgs {
   float* sigma;

@@ -7,10 +7,10 @@
 // monitoring loops where cudaMalloc's implicit device synchronisation would
 // stall unrelated streams, and small tools that hold a state they did not
 // create and so have no clot_mesh (whose workspace comes from cudaMalloc in
-// clot_mesh_create).  This entry point runs the same conjugate-gradient
-// kernel as clot_eta_solve but takes its scratch -- the CG vectors r, p, q,
-// the FP64 reduction partials, the grid-barrier counters and the status words
-// -- from one file-scope static __device__ array.  Every GPU that loads the
+// clot_mesh_create).  This entry point runs the same kernels as clot_eta_solve
+// but takes their scratch -- the residual, the direct solver's work fields and
+// tables or the CG vectors, the FP64 reduction partials, the grid-barrier
+// counters and the status words -- from one file-scope static __device__ array.  Every GPU that loads the
 // library holds that array (about 16.1 MiB) until the process exits.
 //
 // Host code must not use the array's name as a device address (in host code
@@ -26,24 +26,23 @@
 namespace clot {
 
 constexpr long long NOALLOC_MAX_CELLS = 1ll << 20;  // 1,048,576 cells
-constexpr int NOALLOC_MAX_GRID = 4096;              // blocks of the cooperative launch
+constexpr int NOALLOC_MAX_GRID = 2048;              // blocks of the cooperative launch
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 // Layout (bytes): [r | p | q | p2] floats, then partials and reduced scalars
-// (doubles), then the word block: 8 barrier words at +0 (arrival counter,
-// generation, box bounds of the predicted-eta correction; cleared by
-// launch_eta_solve before every launch) and 8 status words at +64 (flags,
+// (doubles), then the word block: 10 barrier words at +0 (arrivals, box bounds
+// of the predicted-eta correction, departures, max theta_B; zero between launches, cleared
+// again by every call) and 8 status words at +128 (flags,
 // iterations, summed iterations, accepted predictions, box corrections and
 // their fallbacks).
 constexpr size_t NA_VEC_BYTES = 4 * NOALLOC_MAX_CELLS * sizeof(float);
-constexpr size_t NA_PART_BYTES = (3 * NOALLOC_MAX_GRID + 8) * sizeof(double);
+constexpr size_t NA_PART_BYTES = 6 * NOALLOC_MAX_GRID * sizeof(double);
 constexpr size_t NA_WORD_BYTES = 256;
-constexpr size_t NA_STATUS_OFF = 64;
+constexpr size_t NA_STATUS_OFF = 128;
 constexpr size_t NA_TOTAL_BYTES = NA_VEC_BYTES + NA_PART_BYTES + NA_WORD_BYTES;
-// The eta kernel uses bar[0..7], status[0..5] and partials[0 .. 3 grid + 5].
-static_assert(8 * sizeof(unsigned) <= NA_STATUS_OFF, "barrier words overlap the status words");
+// The eta kernel uses bar[0..9], status[0..5] and partials[0 .. 6 grid - 1].
+static_assert(10 * sizeof(unsigned) <= NA_STATUS_OFF, "barrier words overlap the status words");
 static_assert(NA_STATUS_OFF + 8 * sizeof(int) <= NA_WORD_BYTES, "status words overflow the word block");
-static_assert((3 * NOALLOC_MAX_GRID + 6) * sizeof(double) <= NA_PART_BYTES, "partials overflow their block");
 static_assert(NA_VEC_BYTES % 256 == 0 && NA_PART_BYTES % 8 == 0, "misaligned scratch blocks");
 
 static __device__ __align__(256) unsigned char g_eta_scratch[NA_TOTAL_BYTES];
@@ -125,6 +124,7 @@ extern "C" int clot_eta_solve_noalloc(const clot_mesh_desc* d, const float* c, i
   a.invPmax = (float)(1.0 / p->Pmax);
   a.tol = (float)p->eta_tol;
   a.atol = (float)p->eta_atol;
+  a.eta_t = (float)p->eta_t;
   a.inner = 1.0f;
   a.maxit = p->eta_maxit;
   a.wait_ns = eta_wait_ns(p->wait_s);
@@ -132,23 +132,48 @@ extern "C" int clot_eta_solve_noalloc(const clot_mesh_desc* d, const float* c, i
   a.maxw = nullptr;
   a.maxw_clear = nullptr;
 
+  // The direct solver, as clot_eta_solve runs it, where its work fields and
+  // cosine tables (rebuilt by every call) fit the scratch beside r; else the
+  // iteration.
+  const long long n4 = (ncell + 3) / 4 * 4, work = (long long)d->ny * d->nz * ((d->nx + 3) / 4 * 4);
+  const long long ty = dct_table_floats(d->ny), tz = d->dim == 3 ? dct_table_floats(d->nz) : 0;
+  const bool direct = dct_applies(a.g) && a.cx > 0.0f && n4 + 2 * work + ty + tz <= 4 * NOALLOC_MAX_CELLS;
   int grid = 0;
-  if (eta_max_grid(&grid) != 0) return na_fail(CLOT_ECUDA, "occupancy query failed");
-  const long long need = (ncell + ETA_BLOCK - 1) / ETA_BLOCK;
-  if (grid > NOALLOC_MAX_GRID) grid = NOALLOC_MAX_GRID;
-  if (grid > need) grid = (int)need;
-  if (grid < 1) grid = 1;
+  if (direct) {
+    a.dct_a = a.r + n4;
+    a.dct_b = a.dct_a + work;
+    float* tab = a.dct_b + work;
+    a.dct_y = tab;
+    a.dct_z = tab + ty;
+    grid = dct_max_grid(a.g);
+    if (grid < 1) return na_fail(CLOT_ECUDA, "occupancy query failed");
+    if (grid > NOALLOC_MAX_GRID) grid = NOALLOC_MAX_GRID;
+  } else {
+    if (eta_max_grid(&grid) != 0) return na_fail(CLOT_ECUDA, "occupancy query failed");
+    const long long need = (ncell + ETA_BLOCK - 1) / ETA_BLOCK;
+    if (grid > NOALLOC_MAX_GRID) grid = NOALLOC_MAX_GRID;
+    if (grid > need) grid = (int)need;
+    if (grid < 1) grid = 1;
+  }
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // The array keeps the previous call's contents.  The counters (status words
   // 1..5) must start at zero; the flags word 0 is left as it is, so that a
   // timeout of an earlier call made without iters (which cannot synchronise to
   // report it) is still reported by the next call given iters.  The barrier
-  // words are cleared by launch_eta_solve; r, p, q and the partials are written
-  // before they are read.
+  // words are cleared below; everything else is written
+  // before it is read.
   if (cudaMemsetAsync(a.status + 1, 0, 5 * sizeof(int), s) != cudaSuccess)
     return na_fail(CLOT_ECUDA, "memset failed");
-  const cudaError_t e = launch_eta_solve(a, grid, s);
+  cudaError_t e = cudaMemsetAsync(a.bar, 0, 10 * sizeof(unsigned), s);
+  if (e != cudaSuccess) return na_fail(CLOT_ECUDA, "memset failed");
+  if (direct) {
+    float* tab = const_cast<float*>(a.dct_y);
+    if ((e = launch_dct_table(d->ny, tab, s)) == cudaSuccess && tz) e = launch_dct_table(d->nz, tab + ty, s);
+    if (e == cudaSuccess) e = launch_eta_dct(a, grid, s);
+  } else {
+    e = launch_eta_solve(a, grid, s);
+  }
   if (e != cudaSuccess) {
     char msg[160];
     snprintf(msg, sizeof(msg), "eta launch: %s", cudaGetErrorString(e));

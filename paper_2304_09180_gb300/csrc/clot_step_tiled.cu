@@ -356,8 +356,9 @@ __device__ __forceinline__ float predict_cell(const StepArgs& A, const float* et
   return r;
 }
 
-// Block maxima of |r| and theta_B into eta_max (float bit patterns; both >= 0).
-__device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[NTH / 32], unsigned* out, int tid) {
+// Block maxima of |r| and theta_B into eta_max (float bit patterns; both >= 0),
+// and of |r| into the word of the block's tile column `tile` when tile >= 0.
+__device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[NTH / 32], unsigned* out, int tile, int tid) {
   for (int o = 16; o > 0; o >>= 1) {
     rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
     bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
@@ -372,7 +373,10 @@ __device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[
       rmax = fmaxf(rmax, red[0][q]);
       bmax = fmaxf(bmax, red[1][q]);
     }
-    if (rmax > 0.0f) atomicMax(out, __float_as_uint(rmax));
+    if (rmax > 0.0f) {
+      atomicMax(out, __float_as_uint(rmax));
+      if (tile >= 0) atomicMax(out + 2 + tile, __float_as_uint(rmax));
+    }
     if (bmax > 0.0f) atomicMax(out + 1, __float_as_uint(bmax));
   }
 }
@@ -524,7 +528,7 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
       bmax = fmaxf(thB, 0.0f);
     }
   }
-  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, tid);
+  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, A.eta_tiles ? G.x0 / BX + (G.nx + BX - 1) / BX * (G.y0 / BY) : -1, tid);
 }
 
 // ---------------------------------------------------------------------------
@@ -697,7 +701,7 @@ __global__ void __launch_bounds__(NTH, 2) species_step_zmarch_kernel(StepArgs A,
     __syncthreads();  // plane k's buffer is refilled by the next iteration's issue
   }
   cp_async_wait_all();
-  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, tid);
+  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, A.eta_tiles ? G.x0 / BX + (G.nx + BX - 1) / BX * (G.y0 / BY) : -1, tid);
 }
 
 template <int DIM, int VEC, bool EXT>
@@ -852,7 +856,7 @@ __device__ __forceinline__ void compute_2d(const StepArgs& A, const EBuf& B, Ens
       bmax = fmaxf(thB, 0.0f);
     }
   }
-  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, tid);
+  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, A.eta_tiles ? G.x0 / BX + (G.nx + BX - 1) / BX * (G.y0 / BY) : -1, tid);
 }
 
 // Five block barriers per item: staged data landed (and the mask cleared),

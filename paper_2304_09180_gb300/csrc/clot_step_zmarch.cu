@@ -245,8 +245,9 @@ __device__ __forceinline__ void zm_w_pass(const ZPlane& B, float* W, int tid, fl
   *reinterpret_cast<float2*>(&W[q]) = w;
 }
 
-// Block maxima of |r| and theta_B into eta_max (float bit patterns; both >= 0).
-__device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[TNT / 32], unsigned* out, int tid) {
+// Block maxima of |r| and theta_B into eta_max (float bit patterns; both >= 0),
+// and of |r| into the word of the block's tile column `tile` when tile >= 0.
+__device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[TNT / 32], unsigned* out, int tile, int tid) {
   for (int o = 16; o > 0; o >>= 1) {
     rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
     bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
@@ -261,7 +262,10 @@ __device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[
       rmax = fmaxf(rmax, red[0][q]);
       bmax = fmaxf(bmax, red[1][q]);
     }
-    if (rmax > 0.0f) atomicMax(out, __float_as_uint(rmax));
+    if (rmax > 0.0f) {
+      atomicMax(out, __float_as_uint(rmax));
+      if (tile >= 0) atomicMax(out + 2 + tile, __float_as_uint(rmax));
+    }
     if (bmax > 0.0f) atomicMax(out + 1, __float_as_uint(bmax));
   }
 }
@@ -476,7 +480,7 @@ __global__ void __launch_bounds__(TNT, 2)
     }
     wsel ^= 1;
   }
-  if (A.predict) block_max2(rmax, bmax, Sm.red, A.eta_max, tid);
+  if (A.predict) block_max2(rmax, bmax, Sm.red, A.eta_max, A.eta_tiles ? (int)(blockIdx.x + gridDim.x * blockIdx.y) : -1, tid);
 }
 
 }  // namespace
