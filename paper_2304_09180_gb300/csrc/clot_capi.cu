@@ -660,23 +660,18 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       }
     }
     A.K.has_sigma = (!(p->flags & CLOT_NO_SIGMA) && f->n_samples > 0) ? 1 : 0;
-    // Strang splitting: the first reaction half-step, cur -> nxt; the
-    // transport then starts from nxt and the step's result lands in cur
-    // (whose state the half-step has consumed).
-    float* c_start = cur;
-    float* c_out = nxt;
+    // Strang splitting: the first reaction half-step, in place; the transport
+    // then starts from its result
     if (strang) {
       StepArgs R = A;
-      R.cin = cur;
-      R.cout = nxt;
+      R.cin = nullptr;
+      R.cout = cur;
       R.eta = ecur;
       R.predict = 0;
       R.cavg = nullptr;
       R.xin = f->ext;  // the extension's rows react in place (null without it)
       R.xout = f->ext;
-      CUDA_OK(traced(m, K_OTHER, s, [&] { return launch_reaction_only(R, s); }));
-      c_start = nxt;
-      c_out = cur;
+      CUDA_OK(traced(m, K_OTHER, s, [&] { return launch_reaction(R, s); }));
     }
     // the extension's rows: transported by their own pass (two with Heun),
     // then reacted in the fused pass's RK4 stages, which writes them back
@@ -712,10 +707,10 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       }
     }
     if (heun && A.K.do_transport) {
-      // two-stage transport: stage 1 (transport only) c_start -> stage
-      // buffer; stage 2 below averages its result with c_start
+      // two-stage transport: stage 1 (transport only) cur -> stage buffer;
+      // stage 2 below averages its result with cur
       StepArgs T = A;
-      T.cin = c_start;
+      T.cin = cur;
       T.cout = m->stage;
       T.eta = ecur;
       T.K.do_reaction = 0;
@@ -725,12 +720,12 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       T.xin = T.xout = nullptr;
       CUDA_OK(traced(m, K_STEP, s, [&] { return launch_species_step_plane(T, s); }));
       A.cin = m->stage;
-      A.cavg = c_start;
+      A.cavg = cur;
     } else {
-      A.cin = c_start;
+      A.cin = cur;
       A.cavg = nullptr;
     }
-    A.cout = c_out;
+    A.cout = nxt;
     A.eta = ecur;
     float* enext = nullptr;
     if (predict) {
@@ -745,7 +740,7 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
     }
     if (run_k1) {
       CUDA_OK(traced(m, K_STEP, s, [&] { return launch_species_step_plane(A, s); }));
-      if (c_out == nxt) std::swap(cur, nxt);
+      std::swap(cur, nxt);
     }
     if (surr) {  // reaction over dt: the network where it applies, RK4 on the fallback list
       const SurrArgs SA = make_surr(m, f, p, mlp, cur, ecur, dt, tol);
@@ -815,10 +810,8 @@ extern "C" int clot_reaction_step(clot_mesh* m, clot_fields* f, const clot_param
   A.K.do_reaction = 1;
   A.K.M = nsub;
   A.K.h = (float)h;
-  A.cin = f->c;
-  A.cout = m->scratch;
-  CUDA_OK(traced(m, K_STEP, s, [&] { return launch_reaction_only(A, s); }));
-  CUDA_OK(cudaMemcpyAsync(f->c, m->scratch, sizeof(float) * CLOT_NS * m->g.pitch, cudaMemcpyDeviceToDevice, s));
+  A.cout = f->c;
+  CUDA_OK(traced(m, K_STEP, s, [&] { return launch_reaction(A, s); }));
   return CLOT_OK;
 }
 

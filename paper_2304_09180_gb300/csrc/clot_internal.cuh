@@ -106,7 +106,6 @@ inline unsigned long long eta_wait_ns(double wait_s) {
 }
 
 // Kernel launchers (defined in the .cu files; all stream-ordered).
-cudaError_t launch_species_step(const StepArgs& a, cudaStream_t s);
 // Tiled fused step (clot_step_tiled.cu): one z plane per block, the plane
 // tile with its halo in shared memory, z neighbours from L2.
 cudaError_t launch_species_step_plane(const StepArgs& a, cudaStream_t s);
@@ -121,7 +120,8 @@ cudaError_t launch_ensemble_step(const StepArgs* chans, const int4* work, int nw
 int ensemble_blocks_per_sm(int dim, bool vec2);
 int tile_x();
 int tile_y();
-cudaError_t launch_reaction_only(const StepArgs& a, cudaStream_t s);
+// Pointwise reaction pass in place on a.cout (clot_step.cu).
+cudaError_t launch_reaction(const StepArgs& a, cudaStream_t s);
 
 // Transport of the inhibitor extension's two rows (clot_step.cu).
 struct ExtArgs {
