@@ -15,6 +15,8 @@
 //                    on injury faces unless the wall exchange is lagged.
 #pragma once
 
+#include <type_traits>
+
 #include "clot_model.cuh"
 
 namespace clot {
@@ -37,6 +39,39 @@ __device__ __forceinline__ float face_flux(float cLL, float cL, float cH, float 
     f = fmaf(Wa * F, cf, f);
   }
   return f;
+}
+
+// face_flux where both outer cells hold values (a cell beyond the mesh holds
+// its neighbour's: the upwind slope is then zero and van Leer keeps the upwind
+// value, as without the cell).  Wa, Wd: hindrance of the advective and of the
+// diffusive flux, pos: F >= 0.  The same roundings as face_flux: the slopes of
+// the two directions are the same differences up to sign.
+__device__ __forceinline__ float face_flux_in(float cLL, float cL, float cH, float cHH, float F, bool pos, float WaF,
+                                              float WdD, int limiter, bool adv) {
+  const float d = cH - cL;
+  float f = -WdD * d;
+  if (adv) {
+    const float cU = pos ? cL : cH;
+    float cf = cU;
+    if (limiter) {
+      const float a = cU - (pos ? cLL : cHH), b = pos ? d : -d;
+      cf = (a * b > 0.0f) ? fmaf(a, __fdividef(b, a + b), cU) : cU;
+    }
+    f = fmaf(WaF, cf, f);
+  }
+  return f;
+}
+
+// Element P of row q of a [rows][pitch] array.  IDX = unsigned: P is a byte
+// offset below 2^32, so that the row's address stays in uniform registers and
+// the access needs no per-thread address arithmetic.
+template <typename IDX, typename T>
+__device__ __forceinline__ T& row_at(T* base, int q, long long pitch, IDX P) {
+  if constexpr (sizeof(IDX) == 4)
+    return *reinterpret_cast<T*>(reinterpret_cast<char*>(const_cast<typename std::remove_const<T>::type*>(base) +
+                                                         q * pitch) + P);
+  else
+    return base[q * pitch + P];
 }
 
 // M classic RK4 steps of size h of the subendothelial E0, C0 (App. B) with the
@@ -75,9 +110,10 @@ __device__ __forceinline__ void wall_ode_rk4(const RxnConst& R, float s1, float&
 // the stored values e0s, c0s (e0n, c0n: the FP32 sums).  With the low words
 // of the deviation form the increments are added in FP64 to the (value, low
 // word) pairs, which are rounded back to two floats each.
+template <bool PLAIN = false>
 __device__ __forceinline__ void wall_store(const StepArgs& A, int fidx, float e0s, float c0s, float e0n, float c0n,
                                            const float (&d)[2]) {
-  if (A.e0lo) {
+  if (!PLAIN && A.e0lo) {
     const double e = ((double)e0s + (double)A.e0lo[fidx]) + (double)d[0];
     const double c = ((double)c0s + (double)A.c0lo[fidx]) + (double)d[1];
     const float eh = (float)e, ch = (float)c;
@@ -106,39 +142,39 @@ __device__ __forceinline__ void wall_store(const StepArgs& A, int fidx, float e0
 //   - the reaction: K.M RK4 steps of K.h (or their exact closed form where
 //     the system reduces to linear activation), the wall exchange coupled in
 //     the stages unless lagged.
-// IDX: the index type of the state arrays (unsigned where the caller has
-// checked that CLOT_NS * pitch < 2^31, for cheaper addressing).  EXT: the
-// inhibitor extension's rows ride along (A.xin after their transport, the
-// result to A.xout), reacted in the same RK4 stages.
-template <typename IDX = long long, bool EXT = false>
+// over: the cell's column lies over the injury patch; gx, gy, k its indices.
+// P: its index in the state arrays (IDX as in row_at).  EXT: the inhibitor
+// extension's rows ride along (A.xin after their transport, the result to
+// A.xout), reacted in the same RK4 stages.  PLAIN: the one-stage step with
+// transport and reaction on, the wall coupled, no deviation form.
+template <typename IDX = long long, bool EXT = false, bool PLAIN = false>
 __device__ __forceinline__ void cell_epilogue(const StepArgs& A, float (&y)[CLOT_NS], const float (&dv)[NT],
-                                              float sig, float etaP, int gx, int gy, int k, IDX P) {
+                                              float sig, float etaP, bool over, int gx, int gy, int k, IDX P) {
   const StepConst& K = A.K;
-  const IDX pitch = (IDX)K.g.pitch;
+  const long long pitch = K.g.pitch;
   float x[2] = {0.0f, 0.0f};
   if (EXT) {
-    x[0] = A.xin[P];
-    x[1] = A.xin[pitch + P];
+    x[0] = row_at(A.xin, 0, pitch, P);
+    x[1] = row_at(A.xin, 1, pitch, P);
   }
   auto store = [&]() {
 #pragma unroll
-    for (int q = 0; q < CLOT_NS; ++q) A.cout[(IDX)q * pitch + P] = y[q];
+    for (int q = 0; q < CLOT_NS; ++q) row_at(A.cout, q, pitch, P) = y[q];
     if (EXT) {
-      A.xout[P] = x[0];
-      A.xout[pitch + P] = x[1];
+      row_at(A.xout, 0, pitch, P) = x[0];
+      row_at(A.xout, 1, pitch, P) = x[1];
     }
   };
-  const bool over = gx >= K.g.i0 && gx <= K.g.i1 && k >= K.g.k0 && k <= K.g.k1;
   const bool wall = over && gy == 0;
   float s1_start = y[CLOT_S1];
-  if (K.do_transport) {
+  if (PLAIN || K.do_transport) {
 #pragma unroll
     for (int t = 0; t < NT; ++t) y[trow(t)] -= K.dtV * dv[t];
     if (K.has_sigma) y[CLOT_ADP] += K.dt * sig;
-    if (A.cavg) {
+    if (!PLAIN && A.cavg) {
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
-        const float ca = __ldg(A.cavg + (IDX)trow(t) * pitch + P);
+        const float ca = __ldg(&row_at(A.cavg, trow(t), pitch, P));
         if (trow(t) == CLOT_S1) s1_start = ca;
         y[trow(t)] = 0.5f * (ca + y[trow(t)]);
       }
@@ -147,7 +183,7 @@ __device__ __forceinline__ void cell_epilogue(const StepArgs& A, float (&y)[CLOT
   const RxnConst& R = K.r;
   int fidx = 0;
   if (wall) fidx = (gx - K.g.i0) + (K.g.i1 - K.g.i0 + 1) * (k - K.g.k0);
-  if (K.wall_lagged && wall && K.do_transport) {
+  if (!PLAIN && K.wall_lagged && wall && K.do_transport) {
     const float e0s = A.e0[fidx], c0s = A.c0[fidx];
     float e0 = e0s, c0 = c0s, d[2];
     const float s1w = (R.Dd * (s1_start + R.s1_ref) + R.kC0m * c0) / (R.Dd + R.kC0p * e0);
@@ -157,13 +193,13 @@ __device__ __forceinline__ void cell_epilogue(const StepArgs& A, float (&y)[CLOT
     wall_ode_rk4(R, y[CLOT_S1] + R.s1_ref, e0, c0, K.dt / (float)K.M, K.M, d);
     wall_store(A, fidx, e0s, c0s, e0, c0, d);
   }
-  if (K.do_reaction) {
+  if (PLAIN || K.do_reaction) {
     const float adhH = (over && gy <= K.g.hadh_jmax) ? R.kadh : 0.0f;
     const float adp = y[CLOT_ADP];
     // k_adp [ADP] / ([ADP]* + [ADP]) is [ADP] itself (+-0) when [ADP] = +-0: skip the division
     const float A1 = (adp != 0.0f) ? R.k_adp * adp / (R.adp_star + adp) : adp;
     const float coh = R.kcohPmax * affinity(R, etaP);
-    const bool wcpl = wall && !K.wall_lagged;
+    const bool wcpl = wall && (PLAIN || !K.wall_lagged);
     if (EXT) {  // the reaction state with the extension's two rows
       float yx[CLOT_NX];
 #pragma unroll
@@ -174,8 +210,8 @@ __device__ __forceinline__ void cell_epilogue(const StepArgs& A, float (&y)[CLOT
         const float e0s = wcpl ? A.e0[fidx] : 0.0f, c0s = wcpl ? A.c0[fidx] : 0.0f;
         float e0 = e0s, c0 = c0s, d[2];
         const float bound = rxn_rk4_dev<CLOT_NX>(R, yx, adhH, A1, coh, wcpl, e0, c0, K.h, K.M, d);
-        if (wcpl) wall_store(A, fidx, e0s, c0s, e0, c0, d);
-        if (bound != 0.0f) A.bound_acc[P] += bound;
+        if (wcpl) wall_store<PLAIN>(A, fidx, e0s, c0s, e0, c0, d);
+        if (bound != 0.0f) row_at(A.bound_acc, 0, 0, P) += bound;
       }
 #pragma unroll
       for (int q = 0; q < CLOT_NS; ++q) y[q] = yx[q];
@@ -188,8 +224,8 @@ __device__ __forceinline__ void cell_epilogue(const StepArgs& A, float (&y)[CLOT
       const float e0s = wcpl ? A.e0[fidx] : 0.0f, c0s = wcpl ? A.c0[fidx] : 0.0f;
       float e0 = e0s, c0 = c0s, d[2];
       const float bound = rxn_rk4_dev(R, y, adhH, A1, coh, wcpl, e0, c0, K.h, K.M, d);
-      if (wcpl) wall_store(A, fidx, e0s, c0s, e0, c0, d);
-      if (bound != 0.0f) A.bound_acc[P] += bound;
+      if (wcpl) wall_store<PLAIN>(A, fidx, e0s, c0s, e0, c0, d);
+      if (bound != 0.0f) row_at(A.bound_acc, 0, 0, P) += bound;
       // the full integration stores its own result: no join with the fast
       // path below while all 15 species are live
       store();

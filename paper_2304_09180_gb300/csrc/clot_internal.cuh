@@ -26,6 +26,11 @@ struct Geom {
   int hadh_jmax;       // H_adh = 1 over the patch for j <= hadh_jmax
 };
 
+// Whether cells (i, ., k) lie over the injury patch.
+__host__ __device__ __forceinline__ bool over_patch(const Geom& g, int i, int k) {
+  return i >= g.i0 && i <= g.i1 && k >= g.k0 && k <= g.k1;
+}
+
 // Reaction constants in FP32 (App. A, App. B, App. E), converted once per call.
 struct RxnConst {
   float kadh, Pmax, kcohPmax, k_adp, adp_star, k_e2, e2_star, n1, n2;
@@ -109,10 +114,9 @@ inline unsigned long long eta_wait_ns(double wait_s) {
 // Tiled fused step (clot_step_tiled.cu): one z plane per block, the plane
 // tile with its halo in shared memory, z neighbours from L2.
 cudaError_t launch_species_step_plane(const StepArgs& a, cudaStream_t s);
-// 3D fused step marching in z with TMA-staged planes (clot_step_zmarch.cu);
-// *used = false (nothing launched) when the mesh or pointers miss its
-// alignment rules (nx % 4, 16-byte bases) or the driver lacks tensor maps.
-cudaError_t launch_zmarch_tma(const StepArgs& a, cudaStream_t s, bool* used);
+// 3D fused step marching in z (clot_step_zmarch.cu), planes staged by TMA where
+// the mesh and the pointers meet its alignment rules, else by asynchronous copies.
+cudaError_t launch_zmarch(const StepArgs& a, cudaStream_t s);
 // Persistent fused step over a work list of (channel, tile column, tile row,
 // plane) items of several meshes (clot_step_tiled.cu).
 cudaError_t launch_ensemble_step(const StepArgs* chans, const int4* work, int nwork, int grid, int dim, bool vec2,

@@ -254,9 +254,11 @@ template <int N = CLOT_NS>
 __device__ __forceinline__ bool rxn_linear_rest(const RxnConst& k, float (&y)[N], float adhH, float A1,
                                                 float coh, bool wall, float h, int M) {
   if (wall || adhH != 0.0f || coh != 0.0f) return false;
-  if (!(y[CLOT_PBA] == 0.0f && y[CLOT_PBSE] == 0.0f && y[CLOT_S1B] == 0.0f && y[CLOT_S2B] == 0.0f &&
-        y[CLOT_E1B] == 0.0f && y[CLOT_E2B] == 0.0f && y[CLOT_C1] == 0.0f && y[CLOT_C2] == 0.0f))
-    return false;
+  // all eight +-0 (one logic operation on the bit patterns per value)
+  const unsigned bits = (__float_as_uint(y[CLOT_PBA]) | __float_as_uint(y[CLOT_PBSE]) | __float_as_uint(y[CLOT_S1B]) |
+                         __float_as_uint(y[CLOT_S2B]) | __float_as_uint(y[CLOT_E1B]) | __float_as_uint(y[CLOT_E2B]) |
+                         __float_as_uint(y[CLOT_C1]) | __float_as_uint(y[CLOT_C2])) & 0x7fffffffu;
+  if (bits != 0u) return false;
   // with the inhibitor extension, E2 stays constant only while kI I E2 = 0
   if (N == CLOT_NX && k.kI * y[N == CLOT_NX ? XINH : 0] * y[CLOT_E2] != 0.0f) return false;
   const float e2 = y[CLOT_E2];

@@ -1,16 +1,11 @@
-// clot_step_tiled.cu -- K1, the fused species step, for the meshes the TMA z
-// march of clot_step_zmarch.cu does not take, and for the ensemble launch:
-//   - species_step_plane_kernel: 2D meshes (and 3D when used plane by plane).
+// clot_step_tiled.cu -- K1, the fused species step, on 2D meshes and for the
+// ensemble launch (3D meshes: the z march of clot_step_zmarch.cu):
+//   - species_step_plane_kernel: 2D meshes.
 //     A block owns a 32 x 8 tile of one plane; the nine species neighbours
 //     read (P^{m,u}, P^{m,a}, P^{b,a}, P^{b,se}, ADP, S1, S2, E1, E2), eta and
 //     eta of the previous step are staged by cp.async with a two-cell halo;
 //     W(theta_T) is computed once per staged cell; each x / y face flux once,
 //     exchanged through shared memory; z neighbours of a 3D plane from L2;
-//   - species_step_zmarch_kernel: 3D meshes whose rows are not 16-byte
-//     multiples (nx % 4 != 0).  A block marches a 32 x 8 tile column through
-//     runs of 12 planes, staging them by cp.async into a four-plane ring,
-//     three ahead; the own column's z neighbours and the flux of the z face
-//     below are carried in registers;
 //   - ensemble_step_kernel: the plane kernel over a work list of (channel,
 //     tile, plane) items of many 3D meshes in one persistent launch;
 //   - ensemble_step2d_kernel: the same for 2D channels, software-pipelined:
@@ -47,15 +42,12 @@ constexpr int SY = BY + 2 * HY;  // 12
 constexpr int SPL = SX * SY;     // 432 cells per staged plane
 constexpr int NST = 9;           // staged species rows 0 .. 8
 
-// Staged tile layout with an x halo of HXT cells (y halo HY): 2 for the
-// cp.async loaders, 4 for the TMA loads (whose x start must be a multiple of
-// 4 floats, 16 bytes).
+// Staged tile layout with an x halo of HXT cells (y halo HY).
 template <int HXT>
 struct Lay {
   static constexpr int HX = HXT, SX = BX + 2 * HXT, SPL = SX * SY;
 };
 using LA = Lay<HX>;
-using LT = Lay<4>;
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
@@ -313,26 +305,6 @@ __device__ __forceinline__ void xy_faces(const StepArgs& A, const float* pl, con
   }
 }
 
-// The rest of a cell's step once all its face fluxes are known: the net
-// outflow of each mobile species present in the block (the others have exactly
-// zero fluxes), then the shared epilogue (transport update, ADP release, the
-// optional Heun average and lagged wall, reaction, store).
-template <bool EXT = false, int SS = -1>
-__device__ __forceinline__ void finish_cell(const StepArgs& A, float (&y)[CLOT_NS], const float (&div)[NT],
-                                            const float (*xf)[BY][BX + 1], const float (*yf)[BY + 1][BX],
-                                            unsigned mask, float sig, float etaP, const TileGeo& G, int k,
-                                            long long P) {
-  const int tx = G.tx, ty = G.ty;
-  float dv[NT];
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    dv[t] = 0.0f;
-    if (A.K.do_transport && species_on<SS>(mask, t))
-      dv[t] = div[t] + (xf[t][ty][tx + 1] - xf[t][ty][tx]) + (yf[t][ty + 1][tx] - yf[t][ty][tx]);
-  }
-  cell_epilogue<long long, EXT>(A, y, dv, sig, etaP, G.gx, G.gy, k, P);
-}
-
 // eta for the next step: linear extrapolation in time, 2 eta - eta_prev, and
 // the exact residual of that guess against the new theta_B (App. A Eq. eta);
 // em/ep are the guesses at k - 1 / k + 1 (used when hm / hp).
@@ -495,7 +467,7 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
       }
     }
     __syncthreads();
-    if (act && K.do_transport) {  // as finish_cell
+    if (act && K.do_transport) {
       const int tx = G.tx, ty = G.ty;
 #pragma unroll
       for (int t = 0; t < NT; ++t)
@@ -519,7 +491,8 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
     for (int q = 0; q < NST; ++q) y[q] = S.plane[q][sc];
 #pragma unroll
     for (int q = NST; q < CLOT_NS; ++q) y[q] = yb[q - NST];
-    cell_epilogue<long long, EXT>(A, y, dv, sig, need_eta ? S.eta[sc] : 0.0f, G.gx, G.gy, k, P);
+    cell_epilogue<long long, EXT>(A, y, dv, sig, need_eta ? S.eta[sc] : 0.0f, over_patch(K.g, G.gx, k), G.gx, G.gy, k,
+                                  P);
     if (A.predict) {
       const float thB = (y[CLOT_PBA] + y[CLOT_PBSE]) * ip;
       const float gm = hm1 ? 2.0f * S.ez[0][0][tid] - S.ez[1][0][tid] : 0.0f;
@@ -528,179 +501,6 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
       bmax = fmaxf(thB, 0.0f);
     }
   }
-  if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, A.eta_tiles ? G.x0 / BX + (G.nx + BX - 1) / BX * (G.y0 / BY) : -1, tid);
-}
-
-// ---------------------------------------------------------------------------
-// 3D fused step marching in z.  A block owns a 32 x 8 tile column and a run
-// of KZ planes.  The planes' tiles (nine species with the halo, eta, eta of
-// the previous step) stream through a ring of four shared-memory buffers by
-// cp.async, three planes ahead of the one being computed, so the loads of
-// plane k + 3 are in flight while plane k computes.  The own-column values of
-// the two planes below stay in registers, and the flux of the z face below a
-// cell is the one computed for the cell underneath one plane earlier: no z
-// neighbour is loaded twice and each z face is computed once.
-constexpr int ZNB = 4;
-struct ZBuf {
-  float c[NST][SPL];
-  float eta[SPL];
-  float etp[SPL];
-};
-struct ZSmem {
-  ZBuf buf[ZNB];
-  float W[SPL];
-  float xf[NT][BY][BX + 1];
-  float yf[NT][BY + 1][BX];
-  float red[2][NTH / 32];
-  unsigned mask;
-};
-
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::); }
-
-template <int VEC>
-__global__ void __launch_bounds__(NTH, 2) species_step_zmarch_kernel(StepArgs A, int KZ) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  ZSmem& S = *reinterpret_cast<ZSmem*>(smraw);
-  const StepConst& K = A.K;
-  const TileGeo G = tile_geo<LA>(K, blockIdx.x, blockIdx.y);
-  const int tid = G.tid, sc = G.sc, nz = G.nz;
-  const long long pitch = G.pitch, sxy = G.sxy;
-  const bool act = G.act;
-  const float ip = K.invPmax;
-  const int kb = blockIdx.z * KZ, ke = min(kb + KZ, nz);
-  const bool need_eta = K.do_reaction || A.predict;
-  const long long P0 = (long long)G.gx + (long long)G.nx * G.gy;  // own cell in plane 0
-
-  auto issue = [&](int k) {  // stage plane k (if it exists and is needed) into its ring buffer
-    if (k < nz && k <= ke + 1) {
-      ZBuf& B = S.buf[k % ZNB];
-      TileLoader<VEC>::load(A, A.cin, pitch, NST, &B.c[0][0], k, G.x0, G.y0, tid);
-      if (need_eta) TileLoader<VEC>::load(A, A.eta, 0, 1, B.eta, k, G.x0, G.y0, tid);
-      if (A.predict) TileLoader<VEC>::load(A, A.eta_prev, 0, 1, B.etp, k, G.x0, G.y0, tid);
-    }
-    cp_async_commit();  // one group per plane, empty or not
-  };
-  issue(kb);
-  issue(kb + 1);
-  issue(kb + 2);
-
-  // own column below the run: mobile species at kb - 1, kb - 2, W and the eta guess at kb - 1
-  float cm1[NT], cm2[NT], fzlo[NT];
-  float Wm1 = 0.0f, gm1 = 0.0f;
-#pragma unroll
-  for (int t = 0; t < NT; ++t) cm1[t] = cm2[t] = fzlo[t] = 0.0f;
-  if (act && kb >= 1) {
-    const long long Q = P0 + (long long)(kb - 1) * sxy;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      cm1[t] = __ldg(A.cin + (long long)trow(t) * pitch + Q);
-      if (kb >= 2) cm2[t] = __ldg(A.cin + (long long)trow(t) * pitch + Q - sxy);
-    }
-    Wm1 = hindrance((cm1[0] + cm1[1] + __ldg(A.cin + CLOT_PBA * pitch + Q) + __ldg(A.cin + CLOT_PBSE * pitch + Q)) *
-                    ip);
-    if (A.predict) gm1 = 2.0f * __ldg(A.eta + Q) - __ldg(A.eta_prev + Q);
-  }
-  float rmax = 0.0f, bmax = 0.0f;
-
-  for (int k = kb; k < ke; ++k) {
-    const long long P = P0 + (long long)k * sxy;
-    const bool hm1 = k >= 1, hm2 = k >= 2, hp1 = k + 1 < nz, hp2 = k + 2 < nz;
-    issue(k + 3);
-    // own-cell values that only this thread needs, meanwhile
-    float yb[CLOT_NS - NST];
-    float sig = 0.0f, Fhi = 0.0f, Flo = 0.0f;
-    if (act) {
-#pragma unroll
-      for (int q = NST; q < CLOT_NS; ++q) yb[q - NST] = __ldg(A.cin + q * pitch + P);
-      if (K.do_transport && K.has_sigma) sig = __ldg(A.sigma + P);
-      if (K.do_transport) {
-        if (hp1) Fhi = __ldg(A.fz + P + sxy);
-        if (k == kb && hm1) Flo = __ldg(A.fz + P);
-      }
-    }
-    const FaceF FF = K.do_transport ? load_face_fluxes(A, G, k) : FaceF{0.0f, 0.0f, 0.0f, 0.0f};
-    if (tid == 0) S.mask = 0u;
-    cp_async_wait_1();  // planes k, k + 1, k + 2 have landed
-    __syncthreads();
-    const ZBuf& B0 = S.buf[k % ZNB];
-    const ZBuf& B1 = S.buf[(k + 1) % ZNB];
-    const ZBuf& B2 = S.buf[(k + 2) % ZNB];
-
-    float c0[NT], cp1[NT], cp2[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      c0[t] = B0.c[trow(t)][sc];
-      cp1[t] = hp1 ? B1.c[trow(t)][sc] : c0[t];
-      cp2[t] = hp2 ? B2.c[trow(t)][sc] : cp1[t];
-    }
-    unsigned bits = w_pass<LA>(K, &B0.c[0][0], S.W, G);
-    if (act && K.do_transport) {
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        const unsigned zb = __float_as_uint(cm2[t]) | __float_as_uint(cm1[t]) | __float_as_uint(cp1[t]) |
-                            __float_as_uint(cp2[t]);
-        bits |= zb ? (1u << t) : 0u;
-      }
-    }
-    mask_or(bits, &S.mask, tid);
-    __syncthreads();
-    const unsigned mask = S.mask;
-
-    float div[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) div[t] = 0.0f;
-    const float WP = S.W[sc];
-    const float Wp = (act && hp1) ? hindrance((cp1[0] + cp1[1] + B1.c[CLOT_PBA][sc] + B1.c[CLOT_PBSE][sc]) * ip) : WP;
-    if (K.do_transport) {
-      xy_faces<LA>(A, &B0.c[0][0], S.W, S.xf, S.yf, mask, G, k, FF);
-      if (act) {
-        const bool advlo = __any_sync(__activemask(), Flo != 0.0f);
-        const bool advhi = __any_sync(__activemask(), Fhi != 0.0f);
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          float lo = 0.0f, hi = 0.0f;
-          if ((mask >> t) & 1u) {
-            if (hm1) {
-              lo = (k == kb) ? face_flux(hm2 ? cm2[t] : cm1[t], cm1[t], c0[t], cp1[t], hm2, hp1, Flo, Wm1, WP, t < 2,
-                                         K.dcoef[t][2], K.limiter, advlo)
-                             : fzlo[t];
-            }
-            if (hp1)
-              hi = face_flux(hm1 ? cm1[t] : c0[t], c0[t], cp1[t], cp2[t], hm1, hp2, Fhi, WP, Wp, t < 2,
-                             K.dcoef[t][2], K.limiter, advhi);
-          }
-          div[t] = hi - lo;
-          fzlo[t] = hi;  // the low face of the cell above
-        }
-      }
-    }
-    __syncthreads();
-
-    if (act) {
-      float y[CLOT_NS];
-#pragma unroll
-      for (int q = 0; q < NST; ++q) y[q] = B0.c[q][sc];
-#pragma unroll
-      for (int q = NST; q < CLOT_NS; ++q) y[q] = yb[q - NST];
-      finish_cell(A, y, div, S.xf, S.yf, mask, sig, need_eta ? B0.eta[sc] : 0.0f, G, k, P);
-      if (A.predict) {
-        const float thB = (y[CLOT_PBA] + y[CLOT_PBSE]) * ip;
-        const float gp = hp1 ? 2.0f * B1.eta[sc] - B1.etp[sc] : 0.0f;
-        rmax = fmaxf(rmax, fabsf(predict_cell<LA>(A, B0.eta, B0.etp, thB, hm1, gm1, hp1, gp, G, P)));
-        bmax = fmaxf(bmax, fmaxf(thB, 0.0f));
-        gm1 = 2.0f * B0.eta[sc] - B0.etp[sc];
-      }
-      // own column shifts down by one plane (old values of plane k)
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        cm2[t] = cm1[t];
-        cm1[t] = c0[t];
-      }
-      Wm1 = WP;
-    }
-    __syncthreads();  // plane k's buffer is refilled by the next iteration's issue
-  }
-  cp_async_wait_all();
   if (A.predict) block_max2(rmax, bmax, S.red, A.eta_max, A.eta_tiles ? G.x0 / BX + (G.nx + BX - 1) / BX * (G.y0 / BY) : -1, tid);
 }
 
@@ -840,7 +640,7 @@ __device__ __forceinline__ void compute_2d(const StepArgs& A, const EBuf& B, Ens
 #pragma unroll
     for (int q = NST; q < CLOT_NS; ++q) y[q] = B.yb[q - NST][tid];
     const float sig = (K.do_transport && K.has_sigma) ? B.sig[tid] : 0.0f;
-    // net outflow of each transported species (as finish_cell, no z faces)
+    // net outflow of each transported species (no z faces)
     float dv[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
@@ -849,7 +649,8 @@ __device__ __forceinline__ void compute_2d(const StepArgs& A, const EBuf& B, Ens
       if (K.do_transport && on)
         dv[t] = 0.0f + (S.xf[t][G.ty][G.tx + 1] - S.xf[t][G.ty][G.tx]) + (S.yf[t][G.ty + 1][G.tx] - S.yf[t][G.ty][G.tx]);
     }
-    cell_epilogue<long long, false>(A, y, dv, sig, need_eta ? B.eta[sc] : 0.0f, G.gx, G.gy, 0, P);
+    cell_epilogue<long long, false>(A, y, dv, sig, need_eta ? B.eta[sc] : 0.0f, over_patch(K.g, G.gx, 0), G.gx, G.gy, 0,
+                                    P);
     if (A.predict) {
       const float thB = (y[CLOT_PBA] + y[CLOT_PBSE]) * K.invPmax;
       rmax = fabsf(predict_cell<LA>(A, B.eta, B.etp, thB, false, 0.0f, false, 0.0f, G, P));
@@ -930,23 +731,6 @@ cudaError_t launch_plane(const StepArgs& a, cudaStream_t s) {
   return a.xin ? launch_plane_t<DIM, VEC, true>(a, s) : launch_plane_t<DIM, VEC, false>(a, s);
 }
 
-constexpr int ZMARCH_KZ = 12;
-template <int VEC>
-cudaError_t launch_zmarch(const StepArgs& a, cudaStream_t s) {
-  const size_t smem = sizeof(ZSmem);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(species_step_zmarch_kernel<VEC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const auto& g = a.K.g;
-  dim3 grid((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, (g.nz + ZMARCH_KZ - 1) / ZMARCH_KZ);
-  species_step_zmarch_kernel<VEC><<<grid, dim3(BX, BY, 1), smem, s>>>(a, ZMARCH_KZ);
-  return cudaGetLastError();
-}
-
 template <int DIM, int VEC>
 cudaError_t launch_ens(const StepArgs* chans, const int4* work, int nwork, int grid, cudaStream_t s) {
   const size_t smem = sizeof(PlaneSmem);
@@ -1006,15 +790,7 @@ int tile_y() { return kTileY; }
 
 cudaError_t launch_species_step_plane(const StepArgs& a, cudaStream_t s) {
   const bool vec2 = (a.K.g.nx % 2) == 0;
-  if (a.K.g.dim == 3) {  // the TMA z march of clot_step_zmarch.cu where its alignment rules hold
-    bool used = false;
-    cudaError_t e = launch_zmarch_tma(a, s, &used);
-    if (e != cudaSuccess || used) return e;
-  }
-  if (a.K.g.dim == 3) {
-    if (a.xin) return cudaErrorNotSupported;  // checked by the caller: the extension takes the TMA z march
-    return vec2 ? launch_zmarch<2>(a, s) : launch_zmarch<1>(a, s);
-  }
+  if (a.K.g.dim == 3) return launch_zmarch(a, s);
   return vec2 ? launch_plane<2, 2>(a, s) : launch_plane<2, 1>(a, s);
 }
 
