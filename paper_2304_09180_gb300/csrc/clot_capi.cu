@@ -40,7 +40,8 @@ struct clot_mesh {
   float* wall_lo;      // [2][max(n_inj, 1)] low words of E0, C0 (CLOT_DEVIATION)
   float* cg;           // [9][ncell] eta solver r, p, q, p2 and the single-reduction CG's five more
   float* eta_ws;       // [2][ncell] eta buffers of the step-to-step prediction
-  unsigned* maxw;      // two sets of (max |r|, max theta_B, max |r| of each 32 x 8 tile column) of the prediction
+  unsigned* maxw;      // three sets of (max |r|, max theta_B, max |r| of each 32 x 8 tile column) of the prediction:
+                       // step n adds to set n mod 3, the eta solve of step n reads the set before and clears the next
   int tiles, nmaxw;    // tile columns recorded, words of a set
   int dct;             // the direct eta solver takes this mesh
   float* dct_tab;      // its cosine tables: y, then z
@@ -56,6 +57,7 @@ struct clot_mesh {
   double pred_t, pred_dt;  // time of the next step, its dt
   float* pred_guess;       // workspace buffer holding the predicted eta of that step
   int pred_sel;            // maxima set the last fused step wrote
+  int one_launch;         // 2D mesh small enough for whole steps in one launch
   int cg_grid, dct_grid;  // blocks of the iterative and of the direct eta solve
   int aux_blocks;
   const float* vfx[2];  // the last two validated (fluxes, dt) sets (double-buffered uploads)
@@ -200,6 +202,11 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
   const long long ntile = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
   m->tiles = ntile <= 4096 ? (int)ntile : 0;  // every block of the eta solve reads them
   m->nmaxw = 2 + m->tiles;
+  // Whole steps in one launch where every tile has a block slot of its own (two
+  // an SM).  Beyond that the launches' cost is small beside the step's, and the
+  // eta solve runs better in blocks of its own size: 1024 x 256 primed channel
+  // 73 us a step launch by launch, 87 in one.
+  m->one_launch = g.dim == 2 && m->dct && ntile <= 2 * eta_sms();
   const long long ty = m->dct ? dct_table_floats(g.ny) : 0, tz = m->dct && g.dim == 3 ? dct_table_floats(g.nz) : 0;
   if (m->dct) {
     m->dct_grid = dct_max_grid(g);
@@ -209,7 +216,9 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
   m->aux_blocks = (int)std::min<long long>(std::max(sms, 1) * 8, std::max<long long>((g.ncell + 255) / 256, 1));
 
-  const size_t npart = (size_t)std::max(6 * std::max(m->cg_grid, m->dct_grid), 8 * m->aux_blocks);
+  const size_t npart = (size_t)std::max<long long>(
+      6 * std::max<long long>(std::max(m->cg_grid, m->dct_grid), g.dim == 2 ? std::min<long long>(ntile, RUN2D_MAX_GRID) : 0),
+      8 * m->aux_blocks);
   if (cudaMalloc(&m->scratch, sizeof(float) * CLOT_NS * g.pitch) != cudaSuccess ||
       cudaMalloc(&m->stage, sizeof(float) * CLOT_NS * g.pitch) != cudaSuccess ||
       cudaMalloc(&m->xws, sizeof(float) * 4 * g.pitch) != cudaSuccess ||
@@ -217,7 +226,7 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
       cudaMalloc(&m->wall_lo, sizeof(float) * 2 * (size_t)std::max(g.n_inj, 1)) != cudaSuccess ||
       cudaMalloc(&m->cg, sizeof(float) * (9 * g.ncell + 32)) != cudaSuccess ||
       cudaMalloc(&m->eta_ws, sizeof(float) * 2 * g.ncell) != cudaSuccess ||
-      cudaMalloc(&m->maxw, sizeof(unsigned) * 2 * m->nmaxw) != cudaSuccess ||
+      cudaMalloc(&m->maxw, sizeof(unsigned) * 3 * m->nmaxw) != cudaSuccess ||
       (m->dct && cudaMalloc(&m->dct_tab, sizeof(float) * (ty + tz)) != cudaSuccess) ||
       cudaMalloc(&m->partials, sizeof(double) * npart) != cudaSuccess ||
       cudaMalloc(&m->dout, sizeof(double) * 8) != cudaSuccess ||
@@ -231,7 +240,7 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
   if (cudaMemset(m->bar, 0, 16 * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(m->status, 0, 8 * sizeof(int)) != cudaSuccess ||
       cudaMemset(m->cg, 0, sizeof(float) * 4 * g.ncell) != cudaSuccess ||
-      cudaMemset(m->maxw, 0, sizeof(unsigned) * 2 * m->nmaxw) != cudaSuccess ||
+      cudaMemset(m->maxw, 0, sizeof(unsigned) * 3 * m->nmaxw) != cudaSuccess ||
       (m->dct && launch_dct_table(g.ny, m->dct_tab, 0) != cudaSuccess) ||
       (tz && launch_dct_table(g.nz, m->dct_tab + ty, 0) != cudaSuccess) ||
       (m->dct && cudaDeviceSynchronize() != cudaSuccess)) {
@@ -538,6 +547,32 @@ extern "C" int clot_species_step_surrogate(clot_mesh* m, clot_fields* f, const c
   return CLOT_OK;
 }
 
+// Whether the step that starts now takes a sample of the ADP release.
+static bool sigma_due(const clot_fields* f, const clot_params* p, double dt) {
+  return f->t + 1e-6 * dt >= (f->n_samples + 1) * p->sigma_dt;
+}
+
+// The sample and the new sigma_release when one is due (Sec. 3.2, Eq. sigma_disc).
+static int sample_sigma(clot_mesh* m, clot_fields* f, const clot_params* p, double dt, cudaStream_t s) {
+  const bool first = f->t_last < 0;
+  if (!first && !sigma_due(f, p, dt)) return CLOT_OK;
+  SigmaArgs sa = make_sigma(m, f, p);
+  if (first) {
+    CUDA_OK(traced(m, K_SIGMA, s, [&] { return launch_sigma_init(sa, s); }));
+    f->t_last = f->t;
+  }
+  if (sigma_due(f, p, dt)) {
+    sa.head = f->n_samples == 0 ? 0 : (f->head + 1) % sa.nslot;
+    sa.nvalid = std::min(f->n_samples + 1, sa.nslot);
+    sa.inv_dt_sample = (float)(1.0 / (f->t - f->t_last));
+    CUDA_OK(traced(m, K_SIGMA, s, [&] { return launch_sigma_sample(sa, s); }));
+    f->head = sa.head;
+    f->n_samples += 1;
+    f->t_last = f->t;
+  }
+  return CLOT_OK;
+}
+
 static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, const clot_params* p, double dt,
                          int nsteps, cudaStream_t s, const clot_mlp* mlp, float tol) {
   if (!m || !fl) return fail(CLOT_EINVAL, "null argument");
@@ -601,9 +636,9 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
   if (cont) {
     ecur = m->pred_guess;
     have_pred = true;
-    sel0 = m->pred_sel ^ 1;
+    sel0 = (m->pred_sel + 1) % 3;
   } else if (predict) {
-    CUDA_OK(cudaMemsetAsync(m->maxw, 0, 2 * m->nmaxw * sizeof(unsigned), s));
+    CUDA_OK(cudaMemsetAsync(m->maxw, 0, 3 * m->nmaxw * sizeof(unsigned), s));
   }
   // Deviation form for the length of the call: the S1, S2 rows and their
   // inlet values shifted by the references (the rates add them back), the
@@ -629,8 +664,68 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
   int last_sel = 0;
   float* cur = f->c;
   float* nxt = f->c_next ? f->c_next : m->scratch;
-  for (int step = 0; step < nsteps; ++step) {
-    const int sel = (step + sel0) & 1;
+  // 2D meshes run whole stretches of steps, up to the next ADP-release sample,
+  // in one launch; per-kernel timing, the surrogate, the inhibitor extension
+  // and meshes or runs the direct eta solver does not take go launch by launch.
+  const bool one_launch = m->one_launch && !m->prof_on && !surr && !ext && run_k1 && (!do_eta || A.ecx > 0.0f);
+  if (one_launch) {
+    Run2d R{};
+    memset(&R, 0, sizeof(R));
+    R.E = make_eta(m, f, p, nullptr);
+    R.stage = m->stage;
+    for (int q = 0; q < 3; ++q) R.eta[q] = ebuf[q];
+    R.maxw = m->maxw;
+    R.nmaxw = m->nmaxw;
+    R.sel = sel0;
+    R.ecur = have_pred ? (ecur == ebuf[1] ? 1 : 2) : 0;
+    R.eprev = 0;
+    R.have_pred = have_pred;
+    R.do_eta = do_eta;
+    R.heun = heun;
+    R.strang = strang;
+    A.eta_res = m->cg;
+    A.eta_tiles = m->tiles;
+    for (int done = 0; done < nsteps;) {
+      if (!(p->flags & CLOT_NO_SIGMA) && (rc = sample_sigma(m, f, p, dt, s))) return rc;
+      A.K.has_sigma = (!(p->flags & CLOT_NO_SIGMA) && f->n_samples > 0) ? 1 : 0;
+      R.nsteps = 0;
+      do {
+        ++R.nsteps;
+        f->t += dt;
+      } while (done + R.nsteps < nsteps && ((p->flags & CLOT_NO_SIGMA) || !sigma_due(f, p, dt)));
+      done += R.nsteps;
+      R.A = A;
+      R.c[0] = cur;
+      R.c[1] = nxt;
+      // where the buffers will be
+      const int sel = R.sel;
+      int ec = R.ecur, ep = R.eprev;
+      for (int q = 0; do_eta && q < R.nsteps; ++q) {
+        const int en = ec == ep ? (ec == 0 ? 1 : 0) : 3 - ec - ep;
+        ep = ec;
+        ec = en;
+      }
+      if (R.nsteps & 1) std::swap(cur, nxt);
+      const bool last = done == nsteps;
+      R.copy_c = last && cur != f->c && !f->c_next;
+      R.copy_eta = last && do_eta && (ep != 0 || ec == 0);
+      CUDA_OK(launch_steps_2d(R, s));
+      if (R.copy_c) cur = f->c;
+      if (R.copy_eta) {
+        if (ec == 0) ec = 3 - ep;
+        ep = 0;
+      }
+      R.ecur = ec;
+      R.eprev = ep;
+      R.have_pred = do_eta;
+      R.sel = (sel + R.nsteps) % 3;
+      last_sel = (sel + R.nsteps - 1) % 3;
+    }
+    ecur = ebuf[R.ecur];
+    eprev = ebuf[R.eprev];
+  }
+  for (int step = 0; step < nsteps && !one_launch; ++step) {
+    const int sel = (step + sel0) % 3;
     last_sel = sel;
     if (do_eta) {
       EtaArgs e = make_eta(m, f, p, cur);
@@ -638,27 +733,12 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       e.inner = 1.0f;  // no over-solve: measured fastest (CG iterations and accepted predictions)
       if (have_pred) {
         e.predicted = 1;
-        e.maxw = m->maxw + m->nmaxw * (sel ^ 1);      // written by the previous fused step
-        e.maxw_clear = m->maxw + m->nmaxw * sel;      // used by this step's fused kernel
+        e.maxw = m->maxw + m->nmaxw * ((sel + 2) % 3);        // written by the previous fused step
+        e.maxw_clear = m->maxw + m->nmaxw * ((sel + 1) % 3);  // for the next one
       }
       CUDA_OK(traced(m, K_ETA, s, [&] { return launch_eta(m, e, s); }));
     }
-    if (!(p->flags & CLOT_NO_SIGMA)) {
-      SigmaArgs sa = make_sigma(m, f, p);
-      if (f->t_last < 0) {
-        CUDA_OK(traced(m, K_SIGMA, s, [&] { return launch_sigma_init(sa, s); }));
-        f->t_last = f->t;
-      }
-      if (f->t + 1e-6 * dt >= (f->n_samples + 1) * p->sigma_dt) {
-        sa.head = f->n_samples == 0 ? 0 : (f->head + 1) % sa.nslot;
-        sa.nvalid = std::min(f->n_samples + 1, sa.nslot);
-        sa.inv_dt_sample = (float)(1.0 / (f->t - f->t_last));
-        CUDA_OK(traced(m, K_SIGMA, s, [&] { return launch_sigma_sample(sa, s); }));
-        f->head = sa.head;
-        f->n_samples += 1;
-        f->t_last = f->t;
-      }
-    }
+    if (!(p->flags & CLOT_NO_SIGMA) && (rc = sample_sigma(m, f, p, dt, s))) return rc;
     A.K.has_sigma = (!(p->flags & CLOT_NO_SIGMA) && f->n_samples > 0) ? 1 : 0;
     // Strang splitting: the first reaction half-step, in place; the transport
     // then starts from its result

@@ -33,8 +33,8 @@ namespace clot {
 __global__ void __launch_bounds__(ETA_BLOCK, 1) eta_cg_kernel(const __grid_constant__ EtaArgs a) {
   const bool v4 = (a.g.nx & 3) == 0 && (a.g.pitch & 3) == 0 && al16(a.c) && al16(a.eta) && al16(a.r) && al16(a.p) &&
                   al16(a.q) && al16(a.p2);
-  Team T{(int)gridDim.x, 0u, 0};
-  EtaOut o{0, 0, false};
+  Team T{(int)gridDim.x, 0u, 0, true};
+  EtaOut o;
   float pr = 0.0f, pb = 0.0f;
   double s_rr = 0.0;
   float s_rmax, s_bmax;
@@ -47,7 +47,15 @@ __global__ void __launch_bounds__(ETA_BLOCK, 1) eta_cg_kernel(const __grid_const
     ok = residual_reduce<ETA_BLOCK>(a, T, v4, s_rr, s_bmax, s_rmax);
   }
   if (ok) ok = eta_iterate<ETA_BLOCK>(a, T, v4, a.predicted != 0, s_rr, s_rmax, s_bmax, o);
-  eta_leave(a, o, ok);
+  eta_note(a, o, ok);
+  team_leave(a);
+}
+
+int eta_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 152;
+  return sms;
 }
 
 int eta_max_grid(int* grid_out) {

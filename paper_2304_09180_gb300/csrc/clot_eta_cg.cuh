@@ -371,10 +371,11 @@ __device__ __forceinline__ bool residual_reduce(const EtaArgs& a, Team& T, bool 
 }
 
 // What a solve did: iterations, whether a prediction was corrected on a box
-// (1) or that was not enough (-1), and whether this block left the team early.
+// (1) or that was not enough (-1), whether this block left the team early, and
+// whether eta was written after the last barrier (another must precede its use).
 struct EtaOut {
-  int it, box;
-  bool gone;
+  int it = 0, box = 0;
+  bool gone = false, sync = false;
 };
 
 // CG until max |r| meets the stopping rule.  predicted: eta and r are the fused
@@ -484,21 +485,24 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
 
     Box B;
     bool use_box = false;
-    const unsigned hx = __ldcg(bw + 3);
+    unsigned w[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) w[d] = __ldcg(bw + d);
+    const unsigned hx = w[3];
     if (s_bmax > 0.0f && pr < 3.0e38f && hx != 0u) {
       const int mx = box_margin(a.cx, pr, (float)stop), my = box_margin(a.cy, pr, (float)stop);
       const int mz = a.g.dim == 3 ? box_margin(a.cz, pr, (float)stop) : 0;
-      B.i0 = max((int)~__ldcg(bw + 0) - mx, 0);
-      B.j0 = max((int)~__ldcg(bw + 1) - my, 0);
-      B.k0 = max((int)~__ldcg(bw + 2) - mz, 0);
+      B.i0 = max((int)~w[0] - mx, 0);
+      B.j0 = max((int)~w[1] - my, 0);
+      B.k0 = max((int)~w[2] - mz, 0);
       B.i1 = min((int)hx - 1 + mx, a.g.nx - 1);
-      B.j1 = min((int)__ldcg(bw + 4) - 1 + my, a.g.ny - 1);
-      B.k1 = min((int)__ldcg(bw + 5) - 1 + mz, a.g.nz - 1);
+      B.j1 = min((int)w[4] - 1 + my, a.g.ny - 1);
+      B.k1 = min((int)w[5] - 1 + mz, a.g.nz - 1);
       use_box = 2 * B.cells() <= a.g.ncell;
     }
     if (use_box) {
       // about eight cells a thread: blocks beyond that would only add arrivals
-      const int want = (int)min((long long)T.nb, max(1ll, B.cells() / (8 * BS)));
+      const int want = T.shrink ? (int)min((long long)T.nb, max(1ll, B.cells() / (8 * BS))) : T.nb;
       if ((int)blockIdx.x >= want) {
         o.gone = true;
         return true;
@@ -624,6 +628,7 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
     }
   }
   if (s_bmax == 0.0f) {  // theta_B = 0 everywhere: eta = 0
+    o.sync = true;
     for_cells(a, T.nb, [&](long long P, int, int, int) { a.eta[P] = 0.0f; });
     return true;
   }
@@ -646,21 +651,23 @@ __device__ __forceinline__ bool prediction_accepted(const EtaArgs& a, float& pr,
   return ok;
 }
 
-// End of a solve, by every block: the status words, and the last block to
-// leave resets the barrier words for the next launch.
-__device__ __forceinline__ void eta_leave(const EtaArgs& a, const EtaOut& o, bool ok) {
+// The status words of a solve.
+__device__ __forceinline__ void eta_note(const EtaArgs& a, const EtaOut& o, bool ok) {
+  if (threadIdx.x != 0 || blockIdx.x != 0 || !ok) return;
+  a.status[1] = o.it;
+  atomicAdd(a.status + 2, o.it);             // iterations summed over solves
+  if (o.box > 0) atomicAdd(a.status + 4, 1);  // predictions corrected on a box
+  if (o.box < 0) atomicAdd(a.status + 5, 1);  // box corrections not enough
+}
+
+// End of a launch, by every block: the last one to leave resets the barrier
+// words for the next launch.
+__device__ __forceinline__ void team_leave(const EtaArgs& a) {
   __syncthreads();
   if (threadIdx.x != 0) return;
-  if (blockIdx.x == 0 && ok) {
-    a.status[1] = o.it;
-    atomicAdd(a.status + 2, o.it);             // iterations summed over solves
-    if (o.box > 0) atomicAdd(a.status + 4, 1);  // predictions corrected on a box
-    if (o.box < 0) atomicAdd(a.status + 5, 1);  // box corrections not enough
-  }
   __threadfence();
-  if (atomicAdd(a.bar + 8, 1u) == gridDim.x - 1) {
+  if (atomicAdd(a.bar + 8, 1u) == gridDim.x - 1)
     for (int q = 0; q < 10; ++q) a.bar[q] = 0u;
-  }
 }
 
 }  // namespace clot

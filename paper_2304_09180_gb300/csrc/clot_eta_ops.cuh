@@ -37,6 +37,7 @@ struct Team {
   int nb;
   unsigned target;
   int half;
+  bool shrink;  // blocks that a solve does not need may leave the launch
 };
 
 // Grid barrier of the team: one arrival per block, whose first thread polls.

@@ -206,6 +206,7 @@ __device__ __forceinline__ int box_margin(float c, float rmax, float stop) {
 constexpr int ETA_BLOCK = 512;
 cudaError_t launch_eta_solve(const EtaArgs& a, int grid, cudaStream_t s);
 int eta_max_grid(int* grid_out);
+int eta_sms();  // SMs of the current device (152 if the query fails)
 
 // Direct solver (clot_eta_dct.cu) for meshes of at most DCT_MAX_NX x DCT_MAX_N
 // (x DCT_MAX_N) cells: its dense transforms cost ny + nz multiply-adds a cell,
@@ -217,6 +218,25 @@ int dct_max_grid(const Geom& g);
 long long dct_table_floats(int n);
 cudaError_t launch_dct_table(int n, float* out, cudaStream_t s);
 cudaError_t launch_eta_dct(const EtaArgs& a, int grid, cudaStream_t s);
+
+// nsteps whole steps of a 2D mesh in one launch (step2d_kernel,
+// clot_step_tiled.cu).  A, E: the step's and the eta solve's arguments without
+// the buffers below, which rotate from step to step.
+struct Run2d {
+  StepArgs A;
+  EtaArgs E;
+  float* c[2];                  // the state and its partner
+  float* stage;                 // first stage of the two-stage transport
+  float* eta[3];                // the caller's eta, two of the workspace
+  unsigned* maxw;               // [3][nmaxw]
+  int nmaxw, sel;               // set the first step adds to
+  int ecur, eprev, have_pred;   // buffers of the first step's eta and of the one before
+  int nsteps, do_eta, heun, strang;
+  int copy_c, copy_eta;         // the result back into c[0] (an odd number of steps), eta back into eta[0]
+  int ntx, nty;
+};
+constexpr int RUN2D_MAX_GRID = 1024;  // blocks (the reduction partials are sized for them)
+cudaError_t launch_steps_2d(Run2d r, cudaStream_t s);
 
 struct SigmaArgs {
   float* sigma;

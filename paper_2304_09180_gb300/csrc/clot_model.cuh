@@ -62,6 +62,18 @@ __device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a,
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// k x / (xs + x), the Hill term of the activation by thrombin (App. A).  Plain
+// plasma holds none, and what first forms is subnormal or close to it: the
+// division's slow path for such numerators (about 500 cycles, in every stage of
+// the integration over the injury) is kept out: zero divides one and keeps
+// itself as the factor, tiny numerators are scaled by a power of two.
+__device__ __forceinline__ float hill_(float k, float x, float xs) {
+  const bool none = x == 0.0f, tiny = fabsf(x) < 1e-20f;
+  const float n = none ? 1.0f : mul_(mul_(k, x), tiny ? 0x1p+64f : 1.0f);
+  return mul_(n / (xs + x), none ? x : tiny ? 0x1p-64f : 1.0f);
+}
+__device__ __forceinline__ double hill_(double k, double x, double xs) { return mul_(k, x) / (xs + x); }
+
 // The injury-face exchange: J, the rates of E0 and C0, and what S1, E1 gain.
 template <typename T>
 __device__ __forceinline__ void wall_rhs(const RxnConst& k, T s1, T e0, T c0, T& fs1, T& fe1, T& fe0, T& fc0) {
@@ -84,7 +96,7 @@ __device__ __forceinline__ void rxn_rhs(const RxnConst& k, const T* y, T adhH, T
   const T c1 = y[CLOT_C1], c2 = y[CLOT_C2];
 
   const T adh = mul_(adhH, (T)k.Pmax - Pbse);
-  const T A = A1 + mul_((T)k.k_e2, e2) / ((T)k.e2_star + e2);
+  const T A = A1 + hill_((T)k.k_e2, e2, (T)k.e2_star);
   const T act = mul_(A, Pmu), ch = mul_(coh, Pma);
   f[CLOT_PMU] = fma_(-adh, Pmu, -act);
   f[CLOT_PMA] = fma_(-adh, Pma, act) - ch;
@@ -262,7 +274,7 @@ __device__ __forceinline__ bool rxn_linear_rest(const RxnConst& k, float (&y)[N]
   // with the inhibitor extension, E2 stays constant only while kI I E2 = 0
   if (N == CLOT_NX && k.kI * y[N == CLOT_NX ? XINH : 0] * y[CLOT_E2] != 0.0f) return false;
   const float e2 = y[CLOT_E2];
-  const float A = A1 + ((e2 != 0.0f) ? k.k_e2 * e2 / (k.e2_star + e2) : e2);  // the A2 term is e2 when e2 = +-0
+  const float A = A1 + hill_(k.k_e2, e2, k.e2_star);
   if (A == 0.0f) return true;
   const float z = -A * h;
   const float q = -z * (1.0f + z * (0.5f + z * ((1.0f / 6.0f) + z * (1.0f / 24.0f))));  // 1 - R(z)

@@ -6,68 +6,10 @@
 
 namespace clot {
 
-// One cell a thread, in place.  Most cells of a mesh hold nothing bound: there
-// the system is linear activation (rxn_linear_rest), which needs neither the
-// fluid-phase factors nor a write beyond P^{m,u}, P^{m,a} -- 13 rows read and
-// at most 2 written instead of 16 and 15.  Every other cell takes the full
-// integration.  256 x 128 x 64 primed duct, 4 of 10 cells not at rest: 114 us,
-// bound by their RK4 arithmetic (all cells integrated into a second buffer that
-// was copied back: 173 us).
-// The closed form multiplies by 1 - R(z), of order z = A h: below 1e-30 that
-// factor would lose bits to the subnormal range, and the integration is taken.
 template <bool EXT>
 __global__ void __launch_bounds__(256, 2) reaction_kernel(const __grid_constant__ StepArgs A) {
-  const StepConst& K = A.K;
-  const RxnConst& R = K.r;
   const long long P = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (P >= K.g.ncell) return;
-  const long long pitch = K.g.pitch;
-  float* c = A.cout + P;
-  constexpr int N = EXT ? CLOT_NX : CLOT_NS;
-  float y[N];
-  const float eta = A.eta[P];
-#pragma unroll
-  for (int q = 0; q < CLOT_NS; ++q)
-    if (q != CLOT_S1 && q != CLOT_S2 && q != CLOT_E1) y[q] = c[q * pitch];
-  if (EXT) {
-    y[EXT ? XINH : 0] = A.xin[P];
-    y[EXT ? XE2I : 0] = A.xin[pitch + P];
-  }
-  const unsigned row = (unsigned)(P / K.g.nx);
-  const int i = (int)(P - (long long)row * K.g.nx), j = (int)(row % K.g.ny), k = (int)(row / K.g.ny);
-  const bool over = i >= K.g.i0 && i <= K.g.i1 && k >= K.g.k0 && k <= K.g.k1;
-  const float adhH = (over && j <= K.g.hadh_jmax) ? R.kadh : 0.0f;
-  const float adp = y[CLOT_ADP], e2 = y[CLOT_E2];
-  const float A1 = R.k_adp * adp / (R.adp_star + adp);
-  const float coh = R.kcohPmax * affinity(R, eta);
-  const bool wall = over && j == 0 && !K.wall_lagged;
-  const float z = (A1 + R.k_e2 * e2 / (R.e2_star + e2)) * K.h;
-  if (z == 0.0f || fabsf(z) > 1e-30f) {
-    const float pmu = y[CLOT_PMU];
-    if (rxn_linear_rest<N>(R, y, adhH, A1, coh, wall, K.h, K.M)) {
-      if (y[CLOT_PMU] != pmu || z != 0.0f) {
-        c[CLOT_PMU * pitch] = y[CLOT_PMU];
-        c[CLOT_PMA * pitch] = y[CLOT_PMA];
-      }
-      return;
-    }
-  }
-  y[CLOT_S1] = c[CLOT_S1 * pitch];
-  y[CLOT_S2] = c[CLOT_S2 * pitch];
-  y[CLOT_E1] = c[CLOT_E1 * pitch];
-  const int fidx = wall ? (i - K.g.i0) + (K.g.i1 - K.g.i0 + 1) * (k - K.g.k0) : 0;
-  const float e0s = wall ? A.e0[fidx] : 0.0f, c0s = wall ? A.c0[fidx] : 0.0f;
-  float e0 = e0s, c0 = c0s, d[2];
-  const float bound = rxn_rk4_dev<N>(R, y, adhH, A1, coh, wall, e0, c0, K.h, K.M, d);
-  if (wall) wall_store(A, fidx, e0s, c0s, e0, c0, d);
-  if (bound != 0.0f) A.bound_acc[P] += bound;
-#pragma unroll
-  for (int q = 0; q < CLOT_NS; ++q)
-    if (q != CLOT_ADP) c[q * pitch] = y[q];
-  if (EXT) {
-    A.xout[P] = y[EXT ? XINH : 0];
-    A.xout[pitch + P] = y[EXT ? XE2I : 0];
-  }
+  if (P < A.K.g.ncell) reaction_cell<EXT>(A, P);
 }
 
 cudaError_t launch_reaction(const StepArgs& a, cudaStream_t s) {

@@ -23,9 +23,11 @@
 // downwind cell (advection) and of the larger theta_T (diffusion, localMax),
 // Sec. 3.2 / App. D; van Leer face values, Gauss-linear diffusion (App. D);
 // boundary table of App. C; reaction terms of App. A and App. B.
+#include <algorithm>
 #include <type_traits>
 
 #include "clot_cell.cuh"
+#include "clot_eta_dct.cuh"
 
 namespace clot {
 namespace {
@@ -63,13 +65,15 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // values of the seven mobile species at k-2, k-1, k+1, k+2 and of P^{b,a},
 // P^{b,se} at k-1, k+1 (for W there), and eta / eta of the previous step on
 // the tile and at k-1, k+1.  The rest of the kernel reads shared memory only.
+template <int DIM>
 struct PlaneSmem {
+  static constexpr int ZT = DIM == 3 ? NTH : 1;  // own-column values of 3D planes
   float plane[NST][SPL];        // rows 0..8 of plane k, halo 2 in x and y
-  float zc[NT][4][NTH];         // mobile species at k-2, k-1, k+1, k+2 (own column)
-  float zb[2][2][NTH];          // P^{b,a}, P^{b,se} at k-1, k+1
+  float zc[NT][4][ZT];         // mobile species at k-2, k-1, k+1, k+2 (own column)
+  float zb[2][2][ZT];          // P^{b,a}, P^{b,se} at k-1, k+1
   float eta[SPL];               // eta on the tile (halo)
   float etp[SPL];               // eta of the previous step on the tile
-  float ez[2][2][NTH];          // [eta, eta_prev][k-1, k+1] (own column)
+  float ez[2][2][ZT];          // [eta, eta_prev][k-1, k+1] (own column)
   float W[SPL];
   float xf[NT][BY][BX + 1];
   float yf[NT][BY + 1][BX];
@@ -112,9 +116,9 @@ struct TileGeo {
 template <class L>
 __device__ __forceinline__ TileGeo tile_geo(const StepConst& K, int bx, int by) {
   TileGeo G;
-  G.tx = threadIdx.x;
-  G.ty = threadIdx.y;
-  G.tid = G.ty * BX + G.tx;
+  G.tid = threadIdx.x + blockDim.x * threadIdx.y;  // 32 x 8 blocks or blocks of 256
+  G.tx = G.tid % BX;
+  G.ty = G.tid / BX;
   G.x0 = bx * BX;
   G.y0 = by * BY;
   G.nx = K.g.nx;
@@ -356,7 +360,7 @@ __device__ __forceinline__ void block_max2(float rmax, float bmax, float (*red)[
 // One 32 x 8 tile (tile column bx, tile row by) of plane k of the mesh A
 // describes.  Called by every thread of the block (it synchronises).
 template <int DIM, int VEC, bool EXT = false>
-__device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int bx, int by, int k) {
+__device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem<DIM>& S, int bx, int by, int k) {
   const StepConst& K = A.K;
   const TileGeo G = tile_geo<LA>(K, bx, by);
   const int tid = G.tid, sc = G.sc, nz = G.nz;
@@ -407,7 +411,7 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
   float sig = 0.0f;
   if (act) {
 #pragma unroll
-    for (int q = NST; q < CLOT_NS; ++q) yb[q - NST] = __ldg(A.cin + q * pitch + P);
+    for (int q = NST; q < CLOT_NS; ++q) yb[q - NST] = __ldcg(A.cin + q * pitch + P);
     if (K.do_transport && K.has_sigma) sig = __ldg(A.sigma + P);
   }
   const FaceF FF = K.do_transport ? load_face_fluxes(A, G, k) : FaceF{0.0f, 0.0f, 0.0f, 0.0f};
@@ -507,8 +511,123 @@ __device__ __forceinline__ void tile_step(const StepArgs& A, PlaneSmem& S, int b
 template <int DIM, int VEC, bool EXT>
 __global__ void __launch_bounds__(NTH, PLANE_MINB) species_step_plane_kernel(StepArgs A) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  PlaneSmem& S = *reinterpret_cast<PlaneSmem*>(smraw);
+  PlaneSmem<DIM>& S = *reinterpret_cast<PlaneSmem<DIM>*>(smraw);
   tile_step<DIM, VEC, EXT>(A, S, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// Any number of whole steps of a 2D mesh in one cooperative launch: per step
+// the eta solve (clot_eta_dct.cuh; nothing to do where the prediction is
+// accepted), with Strang splitting the reaction half-step, the tiles (twice for
+// the two-stage transport), and a grid barrier after each.  A step of a small
+// mesh is a few microseconds of dependent latency; as launches of their own its
+// phases cost as much again each (per step, launch by launch / here: 200 x 40
+// plasma channel 19.2 / 15.7 us, 300 x 64 primed 30 / 24, 320 x 80 second order
+// 36 / 29; the paper's 128 x 32 mesh called step by step 56 / 43).  State, eta and maxima buffers rotate as in the launch
+// sequence of clot_capi.cu; what another block wrote is read after a barrier
+// whose acquire empties the L1, never through the read-only path.
+template <int VEC>
+__global__ void __launch_bounds__(NTH, PLANE_MINB) step2d_kernel(const __grid_constant__ Run2d R) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  PlaneSmem<2>& S = *reinterpret_cast<PlaneSmem<2>*>(smraw);
+  DctSm& D = *reinterpret_cast<DctSm*>(smraw);
+  const int tid = threadIdx.x;  // blocks of 256, as the eta solve counts threads
+  Team T{(int)gridDim.x, 0u, 0, false};
+  int cur = 0, ecur = R.ecur, eprev = R.eprev, sel = R.sel;
+  bool pred = R.have_pred != 0, ok = true;
+  const bool two = R.heun && R.A.K.do_transport;
+  for (int step = 0; step < R.nsteps && ok; ++step) {
+    float* c = R.c[cur];
+    if (R.do_eta) {
+      EtaArgs e = R.E;
+      e.c = c;
+      e.eta = R.eta[ecur];
+      e.predicted = pred;
+      e.maxw = R.maxw + R.nmaxw * (sel == 0 ? 2 : sel - 1);
+      e.maxw_clear = R.maxw + R.nmaxw * (sel == 2 ? 0 : sel + 1);
+      EtaOut o;
+      bool solved;
+      ok = eta_solve_team<NTH>(e, D, T, o, solved);
+      if (ok && solved) {
+        eta_note(e, o, ok);
+        if (o.sync) ok = team_sync(e, T);
+        if (blockIdx.x == 0 && tid >= 2 && tid < 10 && tid != 8) e.bar[tid] = 0u;  // box and maximum of the next solve
+      }
+      if (!ok) break;
+    }
+    const int enext = ecur == eprev ? (ecur == 0 ? 1 : 0) : 3 - ecur - eprev;
+    StepArgs B = R.A;
+    B.eta = R.eta[ecur];
+    if (R.strang) {
+      B.cout = c;
+      for (long long P = (long long)blockIdx.x * NTH + tid; P < B.K.g.ncell; P += (long long)gridDim.x * NTH)
+        reaction_cell<false>(B, P);
+      if (!(ok = team_sync(R.E, T))) break;
+    }
+    for (int ph = two ? 0 : 1; ph < 2 && ok; ++ph) {
+      B.cin = two && ph == 1 ? R.stage : c;
+      B.cout = ph == 1 ? R.c[cur ^ 1] : R.stage;
+      B.cavg = two && ph == 1 ? c : nullptr;
+      B.K.do_reaction = ph == 1 ? R.A.K.do_reaction : 0;
+      B.K.wall_lagged = ph == 1 ? R.A.K.wall_lagged : 0;
+      B.predict = ph == 1 && R.do_eta;
+      B.eta_prev = R.eta[eprev];
+      B.eta_next = R.eta[enext];
+      B.eta_max = R.maxw + R.nmaxw * sel;
+      for (int t = blockIdx.x; t < R.ntx * R.nty; t += gridDim.x) {
+        __syncthreads();  // the block's shared memory is free again
+        tile_step<2, VEC>(B, S, t % R.ntx, t / R.ntx, 0);
+      }
+      ok = team_sync(R.E, T);
+    }
+    if (R.do_eta) {
+      eprev = ecur;
+      ecur = enext;
+      pred = true;
+    }
+    sel = sel == 2 ? 0 : sel + 1;
+    cur ^= 1;
+  }
+  if (ok) {  // results into the caller's buffers
+    const long long t0 = (long long)blockIdx.x * NTH + tid, n = (long long)gridDim.x * NTH;
+    if (R.copy_c) {
+      float* d = R.c[cur ^ 1];
+      const float* s = R.c[cur];
+      const long long tot = (long long)CLOT_NS * R.A.K.g.pitch;
+      if (al16(d) && al16(s)) {
+        for (long long q = t0; q < tot / 4; q += n) st4(d + 4 * q, ld4(s + 4 * q));
+      } else {
+        for (long long q = t0; q < tot; q += n) d[q] = __ldcg(s + q);
+      }
+    }
+    if (R.copy_eta)  // eta of the last step to buffer 0, the prediction out of it
+      for (long long q = t0; q < R.A.K.g.ncell; q += n) {
+        const float g = __ldcg(R.eta[ecur] + q);
+        if (eprev != 0) R.eta[0][q] = __ldcg(R.eta[eprev] + q);
+        if (ecur == 0) R.eta[3 - eprev][q] = g;
+      }
+  }
+  team_leave(R.E);
+}
+
+template <int VEC>
+cudaError_t launch_run2d(const Run2d& r, cudaStream_t s) {
+  const size_t smem = std::max(sizeof(PlaneSmem<2>), sizeof(DctSm));
+  auto* kern = step2d_kernel<VEC>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  static int slots = 0;  // the same on every device the library is built for
+  if (slots == 0) {
+    int dev = 0, sms = 0, per = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NTH, smem)) != cudaSuccess)
+      return e;
+    slots = sms * per;
+  }
+  Run2d copy = r;
+  void* args[] = {&copy};
+  const int grid = std::min(std::min(r.ntx * r.nty, slots), RUN2D_MAX_GRID);
+  return cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(NTH), args, smem, s);
 }
 
 // Ensemble of independent meshes (channels) in one persistent launch: block b
@@ -519,7 +638,7 @@ template <int DIM, int VEC>
 __global__ void __launch_bounds__(NTH, PLANE_MINB) ensemble_step_kernel(const StepArgs* __restrict__ chans,
                                                                const int4* __restrict__ work, int nwork) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  PlaneSmem& S = *reinterpret_cast<PlaneSmem*>(smraw);
+  PlaneSmem<DIM>& S = *reinterpret_cast<PlaneSmem<DIM>*>(smraw);
   __shared__ __align__(16) StepArgs sA;
   const int tid = threadIdx.y * BX + threadIdx.x;
   for (int item = blockIdx.x; item < nwork; item += gridDim.x) {
@@ -712,7 +831,7 @@ __global__ void __launch_bounds__(NTH, PLANE_MINB) ensemble_step2d_kernel(const 
 
 template <int DIM, int VEC, bool EXT>
 cudaError_t launch_plane_t(const StepArgs& a, cudaStream_t s) {
-  const size_t smem = sizeof(PlaneSmem);
+  const size_t smem = sizeof(PlaneSmem<DIM>);
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(species_step_plane_kernel<DIM, VEC, EXT>,
@@ -733,7 +852,7 @@ cudaError_t launch_plane(const StepArgs& a, cudaStream_t s) {
 
 template <int DIM, int VEC>
 cudaError_t launch_ens(const StepArgs* chans, const int4* work, int nwork, int grid, cudaStream_t s) {
-  const size_t smem = sizeof(PlaneSmem);
+  const size_t smem = sizeof(PlaneSmem<DIM>);
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(ensemble_step_kernel<DIM, VEC>,
@@ -769,7 +888,7 @@ cudaError_t launch_ensemble_step(const StepArgs* chans, const int4* work, int nw
 
 int ensemble_blocks_per_sm(int dim, bool vec2) {
   int n = 0;
-  const size_t smem = sizeof(PlaneSmem), smem2 = sizeof(EnsSmem2);
+  const size_t smem = sizeof(PlaneSmem<3>), smem2 = sizeof(EnsSmem2);
   cudaError_t e;
   cudaFuncSetAttribute(ensemble_step_kernel<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaFuncSetAttribute(ensemble_step_kernel<3, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -782,6 +901,13 @@ int ensemble_blocks_per_sm(int dim, bool vec2) {
     e = vec2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ensemble_step2d_kernel<2>, NTH, smem2)
              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ensemble_step2d_kernel<1>, NTH, smem2);
   return e == cudaSuccess ? n : 0;
+}
+
+cudaError_t launch_steps_2d(Run2d r, cudaStream_t s) {
+  const Geom& g = r.A.K.g;
+  r.ntx = (g.nx + BX - 1) / BX;
+  r.nty = (g.ny + BY - 1) / BY;
+  return g.nx % 2 == 0 ? launch_run2d<2>(r, s) : launch_run2d<1>(r, s);
 }
 
 constexpr int kTileX = BX, kTileY = BY;
