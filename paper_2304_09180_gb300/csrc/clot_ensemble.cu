@@ -447,7 +447,7 @@ struct clot_ensemble {
   cudaStream_t cap_stream = nullptr, cap_side[MAXCH - 1] = {};
   cudaEvent_t ev_fork = nullptr, ev_join[MAXCH - 1] = {};
   cudaGraphExec_t graph = nullptr;
-  int graph_grid = -1, graph_nwork = -1, graph_chains = -1;
+  int graph_grid = -1, graph_nwork = -1, graph_chains = -1, graph_eta = -1;
 };
 
 static int efail(int code, const char* fmt, ...) {
@@ -720,7 +720,8 @@ static void fill_versions(clot_ensemble* e, const clot_channel* ch, const clot_p
       A.c0 = f.c0;
       A.bound_acc = f.bound_acc;
       float *ecur, *eprev, *enext;
-      if (n == 0) { ecur = f.eta; eprev = f.eta; enext = W1; }
+      // no eta solve: every step reads the caller's eta
+      if (n == 0 || !do_eta) { ecur = f.eta; eprev = f.eta; enext = W1; }
       else {
         const int m = (n - 1) % 3;
         if (m == 0) { ecur = W1; eprev = f.eta; enext = W2; }
@@ -797,7 +798,9 @@ static cudaError_t launch_version(clot_ensemble* e, int v, bool eta, cudaStream_
 static int ensure_graph(clot_ensemble* e, bool eta) {
   int n = 0;
   while (n < MAXCH && e->cb[n + 1] > e->cb[n]) ++n;
-  if (e->graph && e->graph_grid == e->grid && e->graph_nwork == e->nwork && e->graph_chains == n) return CLOT_OK;
+  if (e->graph && e->graph_grid == e->grid && e->graph_nwork == e->nwork && e->graph_chains == n &&
+      e->graph_eta == eta)
+    return CLOT_OK;
   if (e->graph) {
     cudaGraphExecDestroy(e->graph);
     e->graph = nullptr;
@@ -840,6 +843,7 @@ static int ensure_graph(clot_ensemble* e, bool eta) {
   e->graph_grid = e->grid;
   e->graph_nwork = e->nwork;
   e->graph_chains = n;
+  e->graph_eta = eta;
   return CLOT_OK;
 }
 
