@@ -410,6 +410,29 @@ __global__ void __launch_bounds__(EB) eta_block_cg_kernel(const EtaArgs* __restr
   }
 }
 
+// Channel blockIdx.x: the state and eta of its last step into the buffers its
+// first step started from: one launch for all channels instead of a copy for
+// each.  Bound by launch and memory; its gain was measured with that of
+// upload_versions.
+__global__ void __launch_bounds__(256) results_back_kernel(const StepArgs* __restrict__ first,
+                                                           const StepArgs* __restrict__ last, bool state, bool eta) {
+  const StepArgs& F = first[blockIdx.x];
+  const StepArgs& L = last[blockIdx.x];
+  const long long t = (long long)blockIdx.y * 256 + threadIdx.x, T = (long long)gridDim.y * 256;
+  auto copy = [&](const float* src, float* dst, long long n) {
+    if (src == dst) return;
+    if (((reinterpret_cast<unsigned long long>(src) | reinterpret_cast<unsigned long long>(dst)) & 15u) == 0) {
+      for (long long q = t; q < n / 4; q += T)
+        reinterpret_cast<float4*>(dst)[q] = reinterpret_cast<const float4*>(src)[q];
+      for (long long q = n / 4 * 4 + t; q < n; q += T) dst[q] = src[q];
+    } else {
+      for (long long q = t; q < n; q += T) dst[q] = src[q];
+    }
+  };
+  if (state) copy(L.cout, const_cast<float*>(F.cin), (long long)CLOT_NS * F.K.g.pitch);
+  if (eta) copy(L.eta, const_cast<float*>(F.eta), F.K.g.ncell);
+}
+
 }  // namespace
 }  // namespace clot
 
@@ -442,6 +465,8 @@ struct clot_ensemble {
   EtaArgs* eta_dev = nullptr;    // [7][nchan]
   std::vector<StepArgs> step_host;
   std::vector<EtaArgs> eta_host;
+  std::vector<StepArgs> step_sent;  // what step_dev, eta_dev hold
+  std::vector<EtaArgs> eta_sent;
   std::vector<const float*> vfx, vfy, vfz;
   std::vector<double> vdt;
   cudaStream_t cap_stream = nullptr, cap_side[MAXCH - 1] = {};
@@ -763,12 +788,23 @@ static void fill_versions(clot_ensemble* e, const clot_channel* ch, const clot_p
   }
 }
 
+// The versions onto the device, where they differ from what is there: a run
+// that goes on with the same channels finds its arguments in place, and its
+// first launches need not wait for the stream.  With results_back_kernel, a call
+// of 256 channels (6.8 M cells): 40.93 -> 39.92 ms, runs of one side 0.6 % apart.
 static int upload_versions(clot_ensemble* e, cudaStream_t s) {
+  auto same = [](const auto& a, const auto& b) {
+    return a.size() == b.size() && memcmp(a.data(), b.data(), a.size() * sizeof(a[0])) == 0;
+  };
+  if (same(e->step_host, e->step_sent) && same(e->eta_host, e->eta_sent)) return CLOT_OK;
+  e->step_sent.clear();
   ECUDA(cudaMemcpyAsync(e->step_dev, e->step_host.data(), sizeof(StepArgs) * e->step_host.size(),
                         cudaMemcpyHostToDevice, s));
   ECUDA(cudaMemcpyAsync(e->eta_dev, e->eta_host.data(), sizeof(EtaArgs) * e->eta_host.size(),
                         cudaMemcpyHostToDevice, s));
   ECUDA(cudaStreamSynchronize(s));  // host staging arrays are reused
+  e->step_sent = e->step_host;
+  e->eta_sent = e->eta_host;
   return CLOT_OK;
 }
 
@@ -951,20 +987,14 @@ extern "C" int clot_ensemble_run(clot_ensemble* e, clot_channel* ch, const clot_
     for (int c = 0; c < e->nchan; ++c) ch[c].fields.t += ch[c].dt;
     ++n;
   }
-  // results back into the caller's buffers
-  for (int c = 0; c < e->nchan; ++c) {
-    const Geom& g = e->geom[c];
-    clot_fields& f = ch[c].fields;
-    if (nsteps % 2)
-      ECUDA(cudaMemcpyAsync(f.c, e->scratch + e->off_state[c], sizeof(float) * CLOT_NS * g.pitch,
-                            cudaMemcpyDeviceToDevice, s));
-    if (eta && nsteps >= 2) {
-      const int m = (nsteps - 2) % 3;  // eta used by the last step
-      const float* W1 = e->eta_ws + 2 * e->off_cell[c];
-      const float* used = m == 0 ? W1 : m == 1 ? W1 + g.ncell : f.eta;
-      if (used != f.eta)
-        ECUDA(cudaMemcpyAsync(f.eta, used, sizeof(float) * g.ncell, cudaMemcpyDeviceToDevice, s));
-    }
+  // results back into the caller's buffers: the state after an odd number of
+  // steps, and the eta the last step used where that is not the caller's
+  const bool back_c = nsteps % 2 != 0, back_eta = eta && nsteps >= 2 && (nsteps - 2) % 3 != 2;
+  if (back_c || back_eta) {
+    const int last = nsteps < 2 ? 0 : 1 + (nsteps - 2) % 6;  // version of the last step
+    results_back_kernel<<<dim3(e->nchan, 64), 256, 0, s>>>(e->step_dev, e->step_dev + (size_t)last * e->nchan, back_c,
+                                                           back_eta);
+    ECUDA(cudaGetLastError());
   }
   return CLOT_OK;
 }
