@@ -6,6 +6,8 @@
 //     eta of the previous step are staged by cp.async with a two-cell halo;
 //     W(theta_T) is computed once per staged cell; each x / y face flux once,
 //     exchanged through shared memory; z neighbours of a 3D plane from L2;
+//   - step2d_kernel: small 2D meshes, eta and the fused step of every step of a
+//     call in one cooperative launch;
 //   - ensemble_step_kernel: the plane kernel over a work list of (channel,
 //     tile, plane) items of many 3D meshes in one persistent launch;
 //   - ensemble_step2d_kernel: the same for 2D channels, software-pipelined:
