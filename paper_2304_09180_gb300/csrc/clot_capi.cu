@@ -47,7 +47,7 @@ struct clot_mesh {
   float* dct_tab;      // its cosine tables: y, then z
   double* partials;
   double* dout;        // [8]
-  unsigned* bar;       // [16] grid barrier words, box bounds of the eta correction
+  unsigned* bar;       // [BAR_WORDS] grid barrier words, box bounds of the eta correction
   int* status;         // [8] flags, last eta iterations, summed iterations, accepted predictions, box fixes, box fallbacks
   unsigned long long* scount;  // [4] surrogate fallback counters and list length
   // eta prediction carried from one clot_species_step call to the next
@@ -230,14 +230,14 @@ extern "C" int clot_mesh_create(const clot_mesh_desc* d, clot_mesh** out) {
       (m->dct && cudaMalloc(&m->dct_tab, sizeof(float) * (ty + tz)) != cudaSuccess) ||
       cudaMalloc(&m->partials, sizeof(double) * npart) != cudaSuccess ||
       cudaMalloc(&m->dout, sizeof(double) * 8) != cudaSuccess ||
-      cudaMalloc(&m->bar, sizeof(unsigned) * 16) != cudaSuccess ||
+      cudaMalloc(&m->bar, sizeof(unsigned) * BAR_WORDS) != cudaSuccess ||
       cudaMalloc(&m->status, sizeof(int) * 8) != cudaSuccess ||
       cudaMalloc(&m->scount, sizeof(unsigned long long) * 4) != cudaSuccess) {
     free_mesh(m);
     cudaGetLastError();
     return fail(CLOT_ENOMEM, "device allocation of the mesh workspace failed");
   }
-  if (cudaMemset(m->bar, 0, 16 * sizeof(unsigned)) != cudaSuccess ||
+  if (cudaMemset(m->bar, 0, BAR_WORDS * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(m->status, 0, 8 * sizeof(int)) != cudaSuccess ||
       cudaMemset(m->cg, 0, sizeof(float) * 4 * g.ncell) != cudaSuccess ||
       cudaMemset(m->maxw, 0, sizeof(unsigned) * 3 * m->nmaxw) != cudaSuccess ||
@@ -430,6 +430,7 @@ static EtaArgs make_eta(clot_mesh* m, clot_fields* f, const clot_params* p, cons
   a.cg5 = m->cg + 4 * m->g.ncell;
   a.partials = m->partials;
   a.bar = m->bar;
+  a.own = eta_words(m->bar, 0);
   a.status = m->status;
   a.g = m->g;
   const double cl = p->L_eta * p->L_eta / 4.0;

@@ -362,11 +362,11 @@ __device__ __forceinline__ bool residual_reduce(const EtaArgs& a, Team& T, bool 
   }
   // one barrier for both maxima: |theta_B|'s rides on words of its own
   const unsigned b = __reduce_max_sync(0xffffffffu, __float_as_uint(bmax));
-  if ((threadIdx.x & 31) == 0 && b != 0u) atomicMax(a.bar + 9, b);
+  if ((threadIdx.x & 31) == 0 && b != 0u) atomicMax(a.own + 6, b);
   double sums[1];
   if (!team_reduce<BS, 1>(a, T, {rr}, rmax, sums, s_rmax)) return false;
   s_rr = sums[0];
-  s_bmax = __uint_as_float(__ldcg(a.bar + 9));
+  s_bmax = __uint_as_float(__ldcg(a.own + 6));
   return true;
 }
 
@@ -396,10 +396,10 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
     const float cmax = fmaxf(a.cx, fmaxf(a.cy, a.cz));
     const float thr = (float)(0.5 * stop) / (1.0f + cmax);
     // The bounding box of the cells with |r| > thr, kept as max(~lo) and
-    // max(hi + 1) per axis in bar[2..7].  Only tiles whose maximum the fused
+    // max(hi + 1) per axis in own[0..5].  Only tiles whose maximum the fused
     // step put above thr are swept; a small mesh is swept whole, together with
     // the two inner products that the whole-mesh iteration starts from.
-    unsigned* bw = a.bar + 2;
+    unsigned* bw = a.own;
     Box R{0, a.g.nx - 1, 0, a.g.ny - 1, 0, a.g.nz - 1};
     const bool all = a.tiles == 0 || a.g.ncell <= (1 << 17);
     if (!all) {
@@ -666,8 +666,8 @@ __device__ __forceinline__ void team_leave(const EtaArgs& a) {
   __syncthreads();
   if (threadIdx.x != 0) return;
   __threadfence();
-  if (atomicAdd(a.bar + 8, 1u) == gridDim.x - 1)
-    for (int q = 0; q < 10; ++q) a.bar[q] = 0u;
+  if (atomicAdd(a.bar + 1, 1u) == gridDim.x - 1)
+    for (int q = 0; q < BAR_WORDS; ++q) a.bar[q] = 0u;
 }
 
 }  // namespace clot

@@ -143,6 +143,11 @@ struct ExtArgs {
 };
 cudaError_t launch_ext_transport(const ExtArgs& a, cudaStream_t s);
 
+// Barrier words of the eta solvers: arrivals, departures, then two sets of the
+// words a solve accumulates in (launches of one solve use the first).
+constexpr int ETA_WORDS = 7, BAR_WORDS = 2 + 2 * ETA_WORDS;
+__host__ __device__ __forceinline__ unsigned* eta_words(unsigned* bar, int set) { return bar + 2 + ETA_WORDS * set; }
+
 struct EtaArgs {
   const float* __restrict__ c;  // state (reads Pba, Pbse)
   float* eta;
@@ -153,8 +158,9 @@ struct EtaArgs {
   float* cg5;                   // [5][ncell] second r, two s, two w buffers of the single-reduction CG
                                 // (null: the two-reduction CG)
   double* partials;             // [2][3][gridDim]
-  unsigned* bar;                // [10] arrivals, -, box bounds of the predicted-eta fix (6), departures,
-                                // max theta_B; zero at launch, and again when the launch ends
+  unsigned* bar;                // [BAR_WORDS] arrivals, departures, two sets of solve words; zero at launch, and
+                                // again when the launch ends
+  unsigned* own;                // the solve's set: box bounds of the predicted-eta fix (6), max theta_B
   int* status;                  // [0] flags, [1] iterations, [2] summed iterations, [3] accepted predictions,
                                 // [4] predictions corrected on a box, [5] box corrections that fell back
   Geom g;

@@ -30,9 +30,8 @@ constexpr int NOALLOC_MAX_GRID = 2048;              // blocks of the cooperative
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 // Layout (bytes): [r | p | q | p2] floats, then partials and reduced scalars
-// (doubles), then the word block: 10 barrier words at +0 (arrivals, box bounds
-// of the predicted-eta correction, departures, max theta_B; zero between launches, cleared
-// again by every call) and 8 status words at +128 (flags,
+// (doubles), then the word block: the barrier words at +0 (EtaArgs::bar; zero
+// between launches, cleared again by every call) and 8 status words at +128 (flags,
 // iterations, summed iterations, accepted predictions, box corrections and
 // their fallbacks).
 constexpr size_t NA_VEC_BYTES = 4 * NOALLOC_MAX_CELLS * sizeof(float);
@@ -40,8 +39,8 @@ constexpr size_t NA_PART_BYTES = 6 * NOALLOC_MAX_GRID * sizeof(double);
 constexpr size_t NA_WORD_BYTES = 256;
 constexpr size_t NA_STATUS_OFF = 128;
 constexpr size_t NA_TOTAL_BYTES = NA_VEC_BYTES + NA_PART_BYTES + NA_WORD_BYTES;
-// The eta kernel uses bar[0..9], status[0..5] and partials[0 .. 6 grid - 1].
-static_assert(10 * sizeof(unsigned) <= NA_STATUS_OFF, "barrier words overlap the status words");
+// The eta kernel uses bar[0 .. BAR_WORDS - 1], status[0..5] and partials[0 .. 6 grid - 1].
+static_assert(BAR_WORDS * sizeof(unsigned) <= NA_STATUS_OFF, "barrier words overlap the status words");
 static_assert(NA_STATUS_OFF + 8 * sizeof(int) <= NA_WORD_BYTES, "status words overflow the word block");
 static_assert(NA_VEC_BYTES % 256 == 0 && NA_PART_BYTES % 8 == 0, "misaligned scratch blocks");
 
@@ -109,6 +108,7 @@ extern "C" int clot_eta_solve_noalloc(const clot_mesh_desc* d, const float* c, i
   a.p2 = a.q + NOALLOC_MAX_CELLS;
   a.partials = reinterpret_cast<double*>(b + NA_VEC_BYTES);
   a.bar = reinterpret_cast<unsigned*>(b + NA_VEC_BYTES + NA_PART_BYTES);
+  a.own = eta_words(a.bar, 0);
   a.status = reinterpret_cast<int*>(b + NA_VEC_BYTES + NA_PART_BYTES + NA_STATUS_OFF);
   a.g.dim = d->dim;
   a.g.nx = d->nx;
@@ -165,7 +165,7 @@ extern "C" int clot_eta_solve_noalloc(const clot_mesh_desc* d, const float* c, i
   // before it is read.
   if (cudaMemsetAsync(a.status + 1, 0, 5 * sizeof(int), s) != cudaSuccess)
     return na_fail(CLOT_ECUDA, "memset failed");
-  cudaError_t e = cudaMemsetAsync(a.bar, 0, 10 * sizeof(unsigned), s);
+  cudaError_t e = cudaMemsetAsync(a.bar, 0, BAR_WORDS * sizeof(unsigned), s);
   if (e != cudaSuccess) return na_fail(CLOT_ECUDA, "memset failed");
   if (direct) {
     float* tab = const_cast<float*>(a.dct_y);

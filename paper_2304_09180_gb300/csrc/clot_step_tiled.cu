@@ -546,13 +546,17 @@ __global__ void __launch_bounds__(NTH, PLANE_MINB) step2d_kernel(const __grid_co
       e.predicted = pred;
       e.maxw = R.maxw + R.nmaxw * (sel == 0 ? 2 : sel - 1);
       e.maxw_clear = R.maxw + R.nmaxw * (sel == 2 ? 0 : sel + 1);
+      // A solve adds to its words from zero, and its blocks may read them until
+      // the step's last barrier: the steps alternate between two sets, each
+      // cleared in the step between, a grid barrier from its use on either side.
+      e.own = eta_words(e.bar, step & 1);
+      if (blockIdx.x == 0 && tid < ETA_WORDS) eta_words(e.bar, ~step & 1)[tid] = 0u;
       EtaOut o;
       bool solved;
       ok = eta_solve_team<NTH>(e, D, T, o, solved);
       if (ok && solved) {
         eta_note(e, o, ok);
         if (o.sync) ok = team_sync(e, T);
-        if (blockIdx.x == 0 && tid >= 2 && tid < 10 && tid != 8) e.bar[tid] = 0u;  // box and maximum of the next solve
       }
       if (!ok) break;
     }
