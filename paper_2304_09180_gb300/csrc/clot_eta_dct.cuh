@@ -86,12 +86,16 @@ __device__ __forceinline__ void load_rows(float (&v)[N], const float* p) {
 }
 
 // Forward modes 2 (m0 + .) + par of one tile of 16 column quads.  ld(j): the
-// thread's quad (tid & 15) of row j; st(m, v): its quad of mode m.
+// thread's quad (tid & 15) of row j; st(m, v): its quad of mode m.  sg: the
+// stage of S.a that the next rows go to.  It alternates across the tiles of a
+// block too: the first rows of a tile are copied without a block barrier since
+// the last rows of the tile before were used, and those lie in the other stage.
 template <int BS, int TM, class Ld, class St>
-__device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctSm& S, Ld ld, St st) {
+__device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctSm& S, int& sg, Ld ld, St st) {
   constexpr int GR = BS / 16, MT = TM / GR, NA = TK * TM / 4 / BS, NB = TK / GR;
   const int tid = threadIdx.x, q = tid & 15, g = tid >> 4, n = X.n, H = X.H;
   const int K = par ? n / 2 : (n + 1) / 2;
+  if (K == 0) return;  // n = 1: no odd mode
   const float* Fm = X.F + (long long)par * H * H + m0;
   const float sgn = par ? -1.0f : 1.0f;
   float acc[MT][4];
@@ -101,7 +105,6 @@ __device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctS
     for (int e = 0; e < 4; ++e) acc[u][e] = 0.0f;
   float4 pb[NB], ph[NB];  // rows j and n - 1 - j, folded when they are stored
   auto fetch = [&](int k0) {
-    const int sg = (k0 / TK) & 1;
 #pragma unroll
     for (int u = 0; u < NA; ++u) {
       const int x = tid + u * BS, row = x / (TM / 4), col = 4 * (x % (TM / 4));
@@ -119,7 +122,8 @@ __device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctS
   };
   fetch(0);
   for (int k0 = 0; k0 < K; k0 += TK) {
-    const int sg = (k0 / TK) & 1;
+    const int now = sg;
+    sg ^= 1;
     __syncthreads();  // the last rows are used up
 #pragma unroll
     for (int u = 0; u < NB; ++u)
@@ -134,7 +138,7 @@ __device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctS
     for (int k = 0; k < kn; ++k) {
       const float4 b = *reinterpret_cast<const float4*>(&S.b[0][k][4 * q]);
       float av[MT];
-      load_rows<MT>(av, &S.a[sg][0][k][g * MT]);
+      load_rows<MT>(av, &S.a[now][0][k][g * MT]);
 #pragma unroll
       for (int u = 0; u < MT; ++u) {
         acc[u][0] = fmaf(av[u], b.x, acc[u][0]);
@@ -152,9 +156,10 @@ __device__ __forceinline__ void dct_forward(const Axis& X, int par, int m0, DctS
 }
 
 // Back to rows j0 + . and their mirror rows of one tile of 16 column quads.
-// ld(m): the thread's quad of mode m; st(j, v): its quad of row j.
+// ld(m): the thread's quad of mode m; st(j, v): its quad of row j; sg as in
+// dct_forward.
 template <int BS, int TM, class Ld, class St>
-__device__ __forceinline__ void dct_back(const Axis& X, int j0, DctSm& S, Ld ld, St st) {
+__device__ __forceinline__ void dct_back(const Axis& X, int j0, DctSm& S, int& sg, Ld ld, St st) {
   constexpr int GR = BS / 16, MT = TM / GR, NA = TK * TM / 4 / BS, NB = TK / GR;
   const int tid = threadIdx.x, q = tid & 15, g = tid >> 4, n = X.n, H = X.H;
   const int K = (n + 1) / 2;
@@ -167,7 +172,6 @@ __device__ __forceinline__ void dct_back(const Axis& X, int j0, DctSm& S, Ld ld,
       for (int e = 0; e < 4; ++e) acc[p][u][e] = 0.0f;
   float4 pb[2][NB];
   auto fetch = [&](int k0) {
-    const int sg = (k0 / TK) & 1;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
       const float* Im = X.I + (long long)p * H * H + j0;
@@ -185,7 +189,8 @@ __device__ __forceinline__ void dct_back(const Axis& X, int j0, DctSm& S, Ld ld,
   };
   fetch(0);
   for (int k0 = 0; k0 < K; k0 += TK) {
-    const int sg = (k0 / TK) & 1;
+    const int now = sg;
+    sg ^= 1;
     __syncthreads();  // the last rows are used up
 #pragma unroll
     for (int p = 0; p < 2; ++p)
@@ -201,7 +206,7 @@ __device__ __forceinline__ void dct_back(const Axis& X, int j0, DctSm& S, Ld ld,
       for (int p = 0; p < 2; ++p) {
         const float4 b = *reinterpret_cast<const float4*>(&S.b[p][k][4 * q]);
         float av[MT];
-        load_rows<MT>(av, &S.a[sg][p][k][g * MT]);
+        load_rows<MT>(av, &S.a[now][p][k][g * MT]);
 #pragma unroll
         for (int u = 0; u < MT; ++u) {
           acc[p][u][0] = fmaf(av[u], b.x, acc[p][u][0]);
@@ -316,6 +321,7 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
   float* gb = a.dct_b;
   const bool vr = (nx & 3) == 0 && al16(a.r) && al16(a.eta);  // i0 is a multiple of 4
   const long long rowz = (long long)ny * W4;
+  int sg = 0;  // stage of the shared matrix rows
 
   // ---- y forward: r -> ga
   {
@@ -343,8 +349,8 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
       auto st = [&](int m, float4 v) {
         if (on) st4(dst + (long long)m * W4, v);
       };
-      if (big) dct_forward<BS, 64>(Y, par, m0, S, ld, st);
-      else dct_forward<BS, 32>(Y, par, m0, S, ld, st);
+      if (big) dct_forward<BS, 64>(Y, par, m0, S, sg, ld, st);
+      else dct_forward<BS, 32>(Y, par, m0, S, sg, ld, st);
     }
   }
   if (!team_sync(a, T)) return false;
@@ -365,8 +371,8 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
       auto st = [&](int m, float4 v) {
         if (on) st4(dst + m * rowz, v);
       };
-      if (big) dct_forward<BS, 64>(Z, par, m0, S, ld, st);
-      else dct_forward<BS, 32>(Z, par, m0, S, ld, st);
+      if (big) dct_forward<BS, 64>(Z, par, m0, S, sg, ld, st);
+      else dct_forward<BS, 32>(Z, par, m0, S, sg, ld, st);
     }
     if (!team_sync(a, T)) return false;
     gx = gb;
@@ -402,8 +408,8 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
       auto st = [&](int k, float4 v) {
         if (on) st4(dst + k * rowz, v);
       };
-      if (big) dct_back<BS, 64>(Z, j0, S, ld, st);
-      else dct_back<BS, 32>(Z, j0, S, ld, st);
+      if (big) dct_back<BS, 64>(Z, j0, S, sg, ld, st);
+      else dct_back<BS, 32>(Z, j0, S, sg, ld, st);
     }
     if (!team_sync(a, T)) return false;
   }
@@ -434,8 +440,8 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
         if (i + 2 < w) p[2] = __ldcg(p + 2) + v.z;
         if (i + 3 < w) p[3] = __ldcg(p + 3) + v.w;
       };
-      if (big) dct_back<BS, 64>(Y, j0, S, ld, st);
-      else dct_back<BS, 32>(Y, j0, S, ld, st);
+      if (big) dct_back<BS, 64>(Y, j0, S, sg, ld, st);
+      else dct_back<BS, 32>(Y, j0, S, sg, ld, st);
     }
   }
   return true;
