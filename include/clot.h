@@ -157,8 +157,11 @@ typedef struct {
   double N1, N2, N_A;
   double kC0p, kC0m, kC0cat, kC1p, kC1m, kC1cat, kC2p, kC2m, kC2cat;
   double kS1p, kS1m, kE1p, kE1m, kS2p, kS2m, kE2p, kE2m;
-  double eta_tol;      /* eta solve stops at max|r| <= max(eta_tol max theta_B, eta_atol); */
-  double eta_atol;     /*   max|eta - eta_exact| <= max|r| (M-matrix, unit row sums) */
+  double eta_tol;      /* eta solve: max|eta - eta_exact| <= max(eta_tol max theta_B, eta_atol), down to the */
+  double eta_atol;     /*   rounding of eta.  A start or prediction with max|r| within that bound is kept as it is
+                          (max|eta - eta_exact| <= max|r|: M-matrix, unit row sums); CG stops when its residual
+                          meets it; direct solves repeat while 1e-6 max|r| of their start, which bounds their
+                          rounding errors, exceeds it and the residual still falls */
   double wait_s;       /* bound of each grid-barrier wait of the eta solver, seconds (<= 0: 2 s; at most
                           10 s).  A wait that runs out sets the timeout bit of the device status word and
                           the solver's blocks return; a tiny value makes the waits give up (tests). */
@@ -168,7 +171,7 @@ typedef struct {
   int M_rxn;           /* reaction substeps per step (Sec. 3.2, default 2) */
   int limiter;         /* 0 first-order upwind, 1 van Leer (App. D) */
   int flags;           /* CLOT_NO_* bits */
-  int eta_maxit;       /* iteration cap of the eta solve */
+  int eta_maxit;       /* cap of an eta solve's CG iterations or direct solves */
   const float *pmu_in; /* [ny nz] inlet Dirichlet P^{m,u} (App. C), device */
   const float *s1_in;  /* [ny nz] inlet Dirichlet S1, device */
   const float *s2_in;  /* [ny nz] inlet Dirichlet S2, device */
@@ -202,10 +205,14 @@ int clot_mesh_info(const clot_mesh *mesh, clot_mesh_info_t *out);
  * two validated (fluxes, dt) sets are remembered (double-buffered uploads).
  * Each step's fused kernel also predicts eta for the next step (2 eta - eta of
  * the previous step) with its residual; the next solve accepts it when it
- * meets the stopping rule, else corrects it by CG on the box around the cells
- * whose residual exceeds half the rule's bound (widened by the decay length of
- * the operator) and, if the recomputed residual there still misses the rule,
- * by CG on the whole mesh.  The prediction carries over to the next call when
+ * meets the stopping rule, else corrects it around the cells whose residual
+ * exceeds half the rule's bound, widened by the decay length of the operator.
+ * On meshes of at most 1024 x 512 (x 512) cells with some theta_B above eta_t
+ * (below it g(eta) is zero whatever eta is) the correction is a direct solve, by
+ * cosine transforms along y and z, on the x slab around those cells.  Elsewhere
+ * it is CG on the box around them and, if the recomputed residual next to the
+ * box misses the rule, CG on the whole mesh.
+ * The prediction carries over to the next call when
  * that call continues this one: same fields buffers c and eta, fields->t and
  * dt continuing, and no other call of this library on the mesh in between
  * (they invalidate it).  A caller that changes c or eta itself between calls
@@ -230,7 +237,8 @@ int clot_reaction_step(clot_mesh *mesh, clot_fields *fields, const clot_params *
 
 /* eta solve alone (App. A Eq. eta) from theta_B of fields->c, warm-started from
  * fields->eta; writes fields->eta.  If iters is not NULL the call synchronises,
- * stores the iteration count and reads (and clears) the device status word:
+ * stores the number of CG iterations or direct solves (0: the eta passed in was
+ * kept) and reads (and clears) the device status word:
  * CLOT_ETIMEOUT if a grid-barrier wait of the solver ran out (params->wait_s),
  * in which case fields->eta is only partly solved.
  * Errors: CLOT_EINVAL, CLOT_ECUDA, CLOT_ETIMEOUT. */
@@ -346,9 +354,9 @@ typedef struct {
   int n_step, n_eta, n_sigma, n_other;  /* launches per kind (species step, eta solve, sigma, other) */
   double ms_step, ms_eta, ms_sigma, ms_other; /* summed event time of the timed launches */
   int timed;                             /* launches with event pairs */
-  int eta_iters;                         /* CG iterations summed over the eta solves */
+  int eta_iters;                         /* CG iterations or direct solves summed over the eta solves */
   int eta_accepted;                      /* eta solves that accepted the predicted eta */
-  int eta_box;                           /* eta solves that corrected the predicted eta on a box (App. A, Eq. eta) */
+  int eta_box;                           /* eta solves that corrected the predicted eta on a box or slab (App. A, Eq. eta) */
   int eta_box_fallback;                  /* box corrections that missed the stopping rule and continued on the mesh */
 } clot_profile_t;
 /* Not part of the paper (tracing): start recording; see above. */

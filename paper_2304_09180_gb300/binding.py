@@ -358,7 +358,7 @@ def clot_reaction_step(mesh: Mesh, fields: Fields, params: Params, h: float, nsu
 
 def clot_eta_solve(mesh: Mesh, fields: Fields, params: Params, stream=None) -> int:
     """eta from theta_B of fields.c, warm-started from fields.eta; returns
-    the CG iteration count (synchronises)."""
+    the number of CG iterations or direct solves (synchronises)."""
     f = fields.cstruct()
     it = C.c_int(0)
     _check(lib().clot_eta_solve(mesh.h, C.byref(f), C.byref(params.c), C.byref(it), _stream_ptr(stream)))
@@ -412,7 +412,7 @@ def clot_eta_solve_noalloc(desc: dict, c: torch.Tensor, pitch: int, eta: torch.T
                            stream=None, want_iters=True) -> int | None:
     """eta solve that allocates no device memory (see include/clot.h): for
     callers that cannot call cudaMalloc.  c is the [15, pitch] state, eta the
-    [ncell] warm start / result.  Returns the CG iteration count, or None with
+    [ncell] warm start / result.  Returns the number of CG iterations or direct solves, or None with
     want_iters=False (the call then does not synchronise, and a timeout is
     reported by the next call that asks for the count).  The C side cannot
     check the tensors' sizes or devices, so this wrapper does, before any

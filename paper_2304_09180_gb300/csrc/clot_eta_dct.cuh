@@ -447,8 +447,15 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
   return true;
 }
 
+// Bound of a direct solve's error, relative to max |r|: 5e-7 measured on axes
+// of 512 cells, 3e-7 up to 256.
+constexpr float DCT_ERR = 1e-6f;
+
 // One eta solve by every block of the team (of BS threads): from the fused
-// step's prediction or from the eta passed in, direct or iterated.  solved:
+// step's prediction or from the eta passed in, direct or iterated.  The direct
+// solve repeats until max |eta - eta_exact|, by its error bound, is within the
+// stopping rule's max(tol max theta_B, atol), at most maxit times or until the
+// residual stops falling (the rounding of eta itself).  solved:
 // whether the prediction was not just accepted.  Returns false if a grid
 // barrier gave up.
 template <int BS>
@@ -461,13 +468,16 @@ __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team&
   double s_rr = 0.0;
   if (a.predicted && prediction_accepted(a, rmax, bmax)) return true;
   bool ok = true;
+  float last = 0.0f;  // max |r| before the solve before
   for (int pass = 0;; ++pass) {
     if (pass || !a.predicted) ok = residual_reduce<BS>(a, T, v4, s_rr, bmax, rmax);
     const float stop = fmaxf(a.tol * bmax, a.atol);
     if (!ok || !(bmax > a.eta_t)) break;
     if (a.maxit <= pass || (pass == 0 && rmax <= stop)) break;
+    if (pass && !(rmax < 0.5f * last)) break;  // down to the residual's own rounding
+    last = rmax;
     int i0 = 0, i1 = nx - 1;
-    if (a.predicted && rmax < 3.0e38f) {
+    if (a.predicted && pass == 0 && rmax < 3.0e38f) {
       const float thr = 0.5f * stop / (1.0f + a.cx);
       const int ntx = (nx + 31) >> 5;
       int lo = ntx, hi = -1;
@@ -487,10 +497,13 @@ __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team&
     ok = dct_solve<BS>(a, S, i0, i1, T);
     o.it = pass + 1;
     o.sync = true;
-    o.box = (i0 > 0 || i1 < nx - 1) ? 1 : 0;
-    // a whole-field start on long axes: the transforms' roundings (5e-7 at
-    // 512 cells) refined away by a second solve, on the new residual
-    if (!ok || a.predicted || pass == 1 || max(a.g.ny, a.g.nz) <= 256) break;
+    if (pass == 0) o.box = (i0 > 0 || i1 < nx - 1) ? 1 : 0;
+    // The solve leaves an error of its roundings, below DCT_ERR of max |d|, and
+    // max |d| <= max |r|: another one on the new residual where that may exceed
+    // the rule's bound (starts far from the solution, tight tolerances), and
+    // for a whole-field start on long axes, where the roundings are largest.
+    const bool fine = a.predicted || pass || max(a.g.ny, a.g.nz) <= 256;
+    if (!ok || (fine && DCT_ERR * rmax <= stop)) break;
     if (!(ok = team_sync(a, T))) break;
   }
   if (ok && !(bmax > a.eta_t)) ok = eta_iterate<BS>(a, T, v4, a.predicted != 0, s_rr, rmax, bmax, o);
