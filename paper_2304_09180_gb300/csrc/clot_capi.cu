@@ -459,8 +459,8 @@ static EtaArgs make_eta(clot_mesh* m, clot_fields* f, const clot_params* p, cons
 }
 
 static cudaError_t launch_eta(const clot_mesh* m, const EtaArgs& e, cudaStream_t s) {
-  // the direct solver divides by the x coupling; a run that couples no cells (L_eta = 0) iterates
-  return m->dct && e.cx > 0.0f ? launch_eta_dct(e, m->dct_grid, s) : launch_eta_solve(e, m->cg_grid, s);
+  if (m->dct && dct_coupled(e.cx, e.cy, e.cz)) return launch_eta_dct(e, m->dct_grid, s);
+  return launch_eta_solve(e, m->cg_grid, s);
 }
 
 // Read the device status word (synchronous) and clear its flags: the timeout
@@ -668,7 +668,8 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
   // 2D meshes run whole stretches of steps, up to the next ADP-release sample,
   // in one launch; per-kernel timing, the surrogate, the inhibitor extension
   // and meshes or runs the direct eta solver does not take go launch by launch.
-  const bool one_launch = m->one_launch && !m->prof_on && !surr && !ext && run_k1 && (!do_eta || A.ecx > 0.0f);
+  const bool one_launch = m->one_launch && !m->prof_on && !surr && !ext && run_k1 &&
+                          (!do_eta || dct_coupled(A.ecx, A.ecy, A.ecz));
   if (one_launch) {
     Run2d R{};
     memset(&R, 0, sizeof(R));

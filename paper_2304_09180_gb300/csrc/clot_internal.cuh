@@ -220,6 +220,10 @@ int eta_sms();  // SMs of the current device (152 if the query fails)
 constexpr int DCT_THREADS = 128, DCT_MAX_NX = 1024, DCT_MAX_N = 512;
 __host__ __device__ __forceinline__ int dct_half(int n) { return ((n + 1) / 2 + 63) / 64 * 64; }
 bool dct_applies(const Geom& g);
+// Whether the x coupling is strong enough for it: a mode's x solve works with the
+// ratio (1 + 4 c_y + 4 c_z) / (2 c_x), whose square overflows beyond 1e19.  Weaker
+// couplings (L_eta = 0 among them) are the iteration's.
+inline bool dct_coupled(float cx, float cy, float cz) { return cx > 1e-16f * (1.0f + 4.0f * cy + 4.0f * cz); }
 int dct_max_grid(const Geom& g);
 long long dct_table_floats(int n);
 cudaError_t launch_dct_table(int n, float* out, cudaStream_t s);

@@ -137,7 +137,8 @@ extern "C" int clot_eta_solve_noalloc(const clot_mesh_desc* d, const float* c, i
   // iteration.
   const long long n4 = (ncell + 3) / 4 * 4, work = (long long)d->ny * d->nz * ((d->nx + 3) / 4 * 4);
   const long long ty = dct_table_floats(d->ny), tz = d->dim == 3 ? dct_table_floats(d->nz) : 0;
-  const bool direct = dct_applies(a.g) && a.cx > 0.0f && n4 + 2 * work + ty + tz <= 4 * NOALLOC_MAX_CELLS;
+  const bool direct = dct_applies(a.g) && dct_coupled(a.cx, a.cy, a.cz) &&
+                      n4 + 2 * work + ty + tz <= 4 * NOALLOC_MAX_CELLS;
   int grid = 0;
   if (direct) {
     a.dct_a = a.r + n4;

@@ -50,6 +50,13 @@ def test_error_within_the_rule_from_any_start(mesh, start, eta_tol):
 
 
 @pytest.mark.parametrize("mesh", MESHES)
+@pytest.mark.parametrize("L_eta", [1e-14, 1e-12, 1e-8, 1e-5, 6e-2])
+def test_weak_and_strong_coupling(mesh, L_eta):
+    p = S.params_default(L_eta=L_eta)
+    assert _solve(MESHES[mesh], p, STARTS["zero"], 1e-6) <= max(1e-6, FLOOR)
+
+
+@pytest.mark.parametrize("mesh", MESHES)
 def test_no_iterations_allowed_leaves_eta(mesh):
     import paper_2304_09180_gb300 as clot
     p = S.params_default()
