@@ -278,13 +278,13 @@ __device__ __forceinline__ bool rxn_linear_rest(const RxnConst& k, float (&y)[N]
   if (A == 0.0f) return true;
   const float z = -A * h;
   const float q = -z * (1.0f + z * (0.5f + z * ((1.0f / 6.0f) + z * (1.0f / 24.0f))));  // 1 - R(z)
-  float pmu = y[CLOT_PMU], pma = y[CLOT_PMA];
-  for (int m = 0; m < M; ++m) {
-    pma = fma_(pmu, q, pma);
-    pmu = fma_(-pmu, q, pmu);
-  }
-  y[CLOT_PMU] = pmu;
-  y[CLOT_PMA] = pma;
+  // what P^{m,u} loses is summed apart and added once, as in rxn_rk4: over many
+  // substeps each loss may lie far below the rounding of P^{m,u} itself
+  const float pmu = y[CLOT_PMU];
+  float lost = 0.0f;
+  for (int m = 0; m < M; ++m) lost = fma_(pmu - lost, q, lost);
+  y[CLOT_PMU] = pmu - lost;
+  y[CLOT_PMA] += lost;
   return true;
 }
 
