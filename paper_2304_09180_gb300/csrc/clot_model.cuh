@@ -65,14 +65,15 @@ __device__ __forceinline__ double fma_(double a, double b, double c) { return __
 // k x / (xs + x), the Hill term of the activation by thrombin (App. A).  Plain
 // plasma holds none, and what first forms is subnormal or close to it: the
 // division's slow path for such numerators (about 500 cycles, in every stage of
-// the integration over the injury) is kept out: zero divides one and keeps
-// itself as the factor, tiny numerators are scaled by a power of two.
+// the integration over the injury) is kept out: zero divides one by one (xs may
+// be zero too) and keeps itself as the factor, tiny numerators are scaled by a
+// power of two.
 __device__ __forceinline__ float hill_(float k, float x, float xs) {
   const bool none = x == 0.0f, tiny = fabsf(x) < 1e-20f;
   const float n = none ? 1.0f : mul_(mul_(k, x), tiny ? 0x1p+64f : 1.0f);
-  return mul_(n / (xs + x), none ? x : tiny ? 0x1p-64f : 1.0f);
+  return mul_(n / (none ? 1.0f : xs + x), none ? x : tiny ? 0x1p-64f : 1.0f);
 }
-__device__ __forceinline__ double hill_(double k, double x, double xs) { return mul_(k, x) / (xs + x); }
+__device__ __forceinline__ double hill_(double k, double x, double xs) { return x == 0.0 ? x : mul_(k, x) / (xs + x); }
 
 // The injury-face exchange: J, the rates of E0 and C0, and what S1, E1 gain.
 template <typename T>

@@ -53,3 +53,24 @@ def test_small_increments_add_up(entry, M, Ah):
     tol = (8 + M / 2) * eps * moved
     assert np.all(np.abs(got[O.PMU][rows] - (pmu - moved)) <= 2 * eps * pmu + tol)
     assert np.all(np.abs(got[O.PMA][rows] - (pma + moved)) <= 2 * eps * (pma + moved) + tol)
+
+
+@pytest.mark.parametrize("entry", ["reaction_step", "species_step"])
+@pytest.mark.parametrize("constant", ["adp_star", "e2_star"])
+def test_no_activation_without_its_concentration(entry, constant):
+    """A half-saturation constant of zero with none of the substance: no
+    activation (0, not 0/0), the same bits as with the usual constant."""
+    import torch
+
+    out = []
+    for over in ({}, {constant: 0.0}):
+        clot, p, cfg, mesh, f = _setup(0.0, **over)
+        prm = clot.Params(p, **cfg["inlet"], flags=clot.NO_ETA)
+        if entry == "reaction_step":
+            clot.clot_reaction_step(mesh, f, prm, 1e-5, 2)
+        else:
+            clot.clot_species_step(mesh, f, clot.Fluxes(mesh, **cfg["fluxes"]), prm, cfg["dt"], 1)
+        torch.cuda.synchronize()
+        out.append(f.to_host(mesh)["c"][:, _off_the_floor(cfg)])
+    assert np.all(np.isfinite(out[1]))
+    assert np.array_equal(*out)
