@@ -164,7 +164,11 @@ typedef struct {
                           rounding errors, exceeds it and the residual still falls */
   double wait_s;       /* bound of each grid-barrier wait of the eta solver, seconds (<= 0: 2 s; at most
                           10 s).  A wait that runs out sets the timeout bit of the device status word and
-                          the solver's blocks return; a tiny value makes the waits give up (tests). */
+                          the solver's blocks return; a tiny value makes the waits give up (tests).  The
+                          state of a clot_species_step that timed out is not usable: steps went on from a
+                          partly solved eta or, on small 2D meshes (all steps in one launch), were not
+                          taken although fields.t counts them.  Waits of those launches outside the eta
+                          solve are bounded by 2 s and 0.1 ms for each of M_rxn. */
   double kI;           /* inhibitor extension (fields.ext): association rate of I and fluid-phase E2 */
   double I_in;         /*   and the inlet Dirichlet value of I */
   double S1_ref, S2_ref; /* reference values of S1, S2 under CLOT_DEVIATION (typically the plasma values) */

@@ -685,6 +685,9 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
     R.do_eta = do_eta;
     R.heun = heun;
     R.strang = strang;
+    // A block waits for the cells of others, M RK4 substeps each: a bound far
+    // beyond what those take, whatever bound the caller gives the eta solves.
+    R.wait_ns = 2000000000ull + 100000ull * (unsigned long long)p->M_rxn;
     A.eta_res = m->cg;
     A.eta_tiles = m->tiles;
     for (int done = 0; done < nsteps;) {

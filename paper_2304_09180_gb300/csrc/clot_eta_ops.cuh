@@ -41,10 +41,10 @@ struct Team {
 };
 
 // Grid barrier of the team: one arrival per block, whose first thread polls.
-// Waits are bounded (wait_ns of globaltimer, 2 s by default): a block that
-// gives up sets ST_TIMEOUT and gets false in all its threads; it never arrives
-// again, so every other block's next wait runs out in turn.
-__device__ __forceinline__ bool team_sync(const EtaArgs& a, Team& T) {
+// Waits are bounded (wait_ns of globaltimer, by default that of the eta solves):
+// a block that gives up sets ST_TIMEOUT and gets false in all its threads; it
+// never arrives again, so every other block's next wait runs out in turn.
+__device__ __forceinline__ bool team_sync(const EtaArgs& a, Team& T, unsigned long long wait_ns) {
   __shared__ int ok;
   T.target += (unsigned)T.nb;
   __syncthreads();
@@ -59,7 +59,7 @@ __device__ __forceinline__ bool team_sync(const EtaArgs& a, Team& T) {
       const unsigned long long t = now_ns();
       if (t0 == 0) {
         t0 = t;
-      } else if (t - t0 > a.wait_ns) {
+      } else if (t - t0 > wait_ns) {
         atomicOr(a.status, ST_TIMEOUT);
         ok = 0;
         break;
@@ -69,6 +69,7 @@ __device__ __forceinline__ bool team_sync(const EtaArgs& a, Team& T) {
   __syncthreads();
   return ok != 0;
 }
+__device__ __forceinline__ bool team_sync(const EtaArgs& a, Team& T) { return team_sync(a, T, a.wait_ns); }
 
 // Barrier with a reduction over the team: NS sums s[] and one maximum m (of
 // values >= 0).  Every block writes its partial values before it arrives; after

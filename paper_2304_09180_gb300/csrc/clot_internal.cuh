@@ -244,6 +244,7 @@ struct Run2d {
   int nsteps, do_eta, heun, strang;
   int copy_c, copy_eta;         // the result back into c[0] (an odd number of steps), eta back into eta[0]
   int ntx, nty;
+  unsigned long long wait_ns;   // bound of the waits for other blocks' cells (E.wait_ns: of the eta solves')
 };
 constexpr int RUN2D_MAX_GRID = 1024;  // blocks (the reduction partials are sized for them)
 cudaError_t launch_steps_2d(Run2d r, cudaStream_t s);

@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(NTH, PLANE_MINB) step2d_kernel(const __grid_co
       B.cout = c;
       for (long long P = (long long)blockIdx.x * NTH + tid; P < B.K.g.ncell; P += (long long)gridDim.x * NTH)
         reaction_cell<false>(B, P);
-      if (!(ok = team_sync(R.E, T))) break;
+      if (!(ok = team_sync(R.E, T, R.wait_ns))) break;
     }
     for (int ph = two ? 0 : 1; ph < 2 && ok; ++ph) {
       B.cin = two && ph == 1 ? R.stage : c;
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(NTH, PLANE_MINB) step2d_kernel(const __grid_co
         __syncthreads();  // the block's shared memory is free again
         tile_step<2, VEC>(B, S, t % R.ntx, t / R.ntx, 0);
       }
-      ok = team_sync(R.E, T);
+      ok = team_sync(R.E, T, R.wait_ns);
     }
     if (R.do_eta) {
       eprev = ecur;
