@@ -252,7 +252,7 @@ __device__ __forceinline__ void reaction_cell(const StepArgs& A, long long P) {
   float* c = A.cout + P;
   constexpr int N = EXT ? CLOT_NX : CLOT_NS;
   float y[N];
-  const float eta = A.eta[P];
+  const float eta = __ldcg(A.eta + P);  // written by other blocks of the same launch where steps share one
 #pragma unroll
   for (int q = 0; q < CLOT_NS; ++q)
     if (q != CLOT_S1 && q != CLOT_S2 && q != CLOT_E1) y[q] = c[q * pitch];
