@@ -69,11 +69,13 @@ def test_no_iterations_allowed_leaves_eta(mesh):
     assert np.all(f.eta.cpu().numpy() == 0.25)
 
 
-@pytest.mark.parametrize("name", ["duct_300x24x20", "duct_203x67x45", "channel_301x40", "channel_900x72"])
+@pytest.mark.parametrize("name", ["duct_300x24x20", "duct_203x67x45", "channel_301x40", "channel_900x72",
+                                  "duct_60x256x256", "duct_61x320x330"])
 @pytest.mark.parametrize("eta_tol", [1e-6, 1e-9])
 def test_predicted_eta_of_a_step(name, eta_tol):
     """The eta a step used, solved from the prediction of the step before: the
-    clot keeps the slab that is corrected inside the mesh."""
+    clot keeps the slab that is corrected inside the mesh.  The last two lie on
+    either side of the rule that leaves wide cross sections to CG on a box."""
     import torch
 
     import paper_2304_09180_gb300 as clot
