@@ -386,6 +386,11 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
                                             float s_rmax, float s_bmax, EtaOut& o) {
   const long long pitch = a.g.pitch;
   const double stop = (double)a.inner * fmax((double)a.tol * s_bmax, (double)a.atol);
+  if (s_bmax == 0.0f) {  // theta_B = 0 everywhere: eta = 0, whatever r holds
+    o.sync = true;
+    for_cells(a, T.nb, [&](long long P, int, int, int) { a.eta[P] = 0.0f; });
+    return true;
+  }
   double s_del = 0.0;
   if (predicted) {
     // Core threshold: a cell just inside the box edge with |r| <= thr gets a
@@ -489,7 +494,7 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
 #pragma unroll
     for (int d = 0; d < 6; ++d) w[d] = __ldcg(bw + d);
     const unsigned hx = w[3];
-    if (s_bmax > 0.0f && pr < 3.0e38f && hx != 0u) {
+    if (pr < 3.0e38f && hx != 0u) {
       const int mx = box_margin(a.cx, pr, (float)stop), my = box_margin(a.cy, pr, (float)stop);
       const int mz = a.g.dim == 3 ? box_margin(a.cz, pr, (float)stop) : 0;
       B.i0 = max((int)~w[0] - mx, 0);
@@ -626,11 +631,6 @@ __device__ __forceinline__ bool eta_iterate(const EtaArgs& a, Team& T, bool v4, 
       s_rr = sums[0];
       s_del = sums[1];
     }
-  }
-  if (s_bmax == 0.0f) {  // theta_B = 0 everywhere: eta = 0
-    o.sync = true;
-    for_cells(a, T.nb, [&](long long P, int, int, int) { a.eta[P] = 0.0f; });
-    return true;
   }
   if (a.cg5)
     return cg_single_reduction<BS>(a, T, v4 && al16(a.cg5) && (a.g.ncell & 3) == 0, s_rr, s_del, s_rmax, stop, o.it);

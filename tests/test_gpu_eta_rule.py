@@ -93,3 +93,18 @@ def test_predicted_eta_of_a_step(name, eta_tol):
     th = _theta(c, p, d)
     got = f.eta.double().cpu().numpy()
     assert np.max(np.abs(got - exact_eta(d, p, th).reshape(-1))) <= max(2 * eta_tol, FLOOR) * np.max(th)
+
+
+@pytest.mark.parametrize("name", ["duct_45x24x20", "channel_131x40", "channel_1030x20"])
+def test_nothing_bound_over_steps(name):
+    """Transport alone of plain plasma: eta is zero in every step, from any start."""
+    import paper_2304_09180_gb300 as clot
+    p = S.params_default(eta_tol=1e-6)
+    cfg = S.config(name, p)
+    d = cfg["desc"]
+    mesh = clot.Mesh(d)
+    f = clot.Fields.from_host(mesh, p, *S.plasma_state(d, p, seed=2), eta=0.1 * np.ones(mesh.ncell))
+    prm = clot.Params(p, **cfg["inlet"], flags=clot.NO_REACTION)
+    for n in (1, 2, 3):
+        clot.clot_species_step(mesh, f, clot.Fluxes(mesh, **cfg["fluxes"]), prm, cfg["dt"], n)
+        assert np.all(f.eta.cpu().numpy() == 0.0)
