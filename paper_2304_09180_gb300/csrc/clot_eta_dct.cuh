@@ -31,8 +31,8 @@
 // max|r| bounds the correction (A is an M-matrix and A exp(-mu |x|) >= 0), so
 // the cells next to the slab keep a residual within the stopping rule.
 //
-// Where that is faster (box_cg_cheaper) the prediction is corrected by CG on a box
-// instead.  Where no theta_B exceeds eta_t the kernel iterates too (clot_eta_cg.cuh):
+// Where that is faster (direct_ns, box_cg_ns) the prediction is corrected by CG on
+// a box instead.  Where no theta_B exceeds eta_t the kernel iterates too (clot_eta_cg.cuh):
 // eta <= max theta_B, so the affinity g(eta) is zero in every cell whatever the
 // solve returns, and what it returns is the iterate that first meets the
 // stopping rule -- one or two iterations from a prediction.
@@ -448,26 +448,28 @@ __device__ __forceinline__ bool dct_solve(const EtaArgs& a, DctSm& S, int i0, in
   return true;
 }
 
-// Whether CG on a box corrects a 3D prediction faster than the direct solve: on
-// wide cross sections, whose dense transforms cost ny + nz multiply-adds for
-// every cell of the slab, when cells couple weakly, so that few iterations are
-// enough (in 2D the transforms never cost what CG's barriers do).
-// w, rows: columns and rows of the mesh that the correction reaches.  Times in
-// ns, fitted to (eta a step, direct / CG, us; h in um, 256 x n x n primed ducts):
+// Times, in ns, of correcting a 3D prediction by the direct solve on a slab of w
+// columns, and by CG on a box of w columns and the given rows.  CG is faster on
+// wide cross sections, whose dense transforms cost ny + nz multiply-adds for every
+// cell of the slab, when cells couple weakly, so that few iterations are enough
+// (in 2D the transforms never cost what CG's barriers do).  Fitted to (eta a step,
+// direct / CG, us; h in um, 256 x n x n primed ducts):
 //   h 1.5   n 128: 78 / 375   256: 258 / 375   320: 465 / 386   384: 667 / 421   (128 x 512 x 512: 1306 / 322)
 //   h 3.0   n 128: 55 / 115   192:  94 / 104   256: 161 / 118   320: 276 / 116
 //   h 0.75  n 128: 152 / 1342                  256: 573 / 5209  320: 1153 / 8312
 // CG takes 0.6 of its bound, sqrt(condition) / 2 ln(2 max|r| / stop) iterations,
 // each of two barriers and a pass over the box.
-__device__ __forceinline__ bool box_cg_cheaper(const EtaArgs& a, float rmax, float stop, int w, int rows) {
+constexpr float CG_START_NS = 4.0e4f, CG_ITER_NS = 6.0e4f;
+__device__ __forceinline__ float direct_ns(const EtaArgs& a, int w) {
   auto dense = [](int n) {  // multiply-adds a cell along an axis of n, whole tiles counted
     const int half = (n + 1) >> 1;
     return n > 1 ? 4.0f * (float)((half + 31) & ~31) * (float)((half + 63) & ~63) / (float)n : 0.0f;
   };
+  return 3.0e4f + (float)w * (float)a.g.ny * (float)a.g.nz * (dense(a.g.ny) + dense(a.g.nz)) / 1.7e4f;
+}
+__device__ __forceinline__ float box_cg_ns(const EtaArgs& a, float rmax, float stop, int w, int rows) {
   const float its = fmaxf(0.3f * sqrtf(1.0f + 4.0f * (a.cx + a.cy + a.cz)) * logf(2.0f * rmax / stop), 1.0f);
-  const float cols = (float)w * (float)a.g.nz;
-  const float direct = 3.0e4f + cols * (float)a.g.ny * (dense(a.g.ny) + dense(a.g.nz)) / 1.7e4f;
-  return 4.0e4f + its * (6.0e4f + 0.018f * cols * (float)rows) < direct;
+  return CG_START_NS + its * (CG_ITER_NS + 0.018f * (float)w * (float)rows * (float)a.g.nz);
 }
 
 // Bound of a direct solve's error, relative to max |r|: 5e-7 measured on axes
@@ -503,13 +505,11 @@ __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team&
     if (a.predicted && pass == 0 && rmax < 3.0e38f) {
       const float thr = 0.5f * stop / (1.0f + a.cx);
       const int ntx = (nx + 31) >> 5;
-      int lo = ntx, hi = -1, ylo = a.g.ny, yhi = -1;
+      int lo = ntx, hi = -1;
       for (int t = threadIdx.x & 31; t < a.tiles; t += 32)
         if (__uint_as_float(__ldcg(a.maxw + 2 + t)) > thr) {
           lo = min(lo, t % ntx);
           hi = max(hi, t % ntx);
-          ylo = min(ylo, t / ntx);
-          yhi = max(yhi, t / ntx);
         }
       lo = __reduce_min_sync(0xffffffffu, lo);
       hi = __reduce_max_sync(0xffffffffu, hi);
@@ -517,11 +517,18 @@ __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team&
         const int mx = box_margin(a.cx, rmax, stop);
         i0 = max(32 * lo - mx, 0) & ~3;
         i1 = min((32 * hi + 31 + mx) | 3, nx - 1);  // whole quads where nx has them
-        if (a.g.dim == 3) {
+        const float direct = a.g.dim == 3 ? direct_ns(a, i1 - i0 + 1) : 0.0f;
+        if (direct > CG_START_NS + CG_ITER_NS) {
+          int ylo = a.g.ny, yhi = -1;
+          for (int t = threadIdx.x & 31; t < a.tiles; t += 32)
+            if (__uint_as_float(__ldcg(a.maxw + 2 + t)) > thr) {
+              ylo = min(ylo, t / ntx);
+              yhi = max(yhi, t / ntx);
+            }
           const int my = box_margin(a.cy, rmax, stop);
           ylo = max(8 * __reduce_min_sync(0xffffffffu, ylo) - my, 0);
           yhi = min(8 * __reduce_max_sync(0xffffffffu, yhi) + 7 + my, a.g.ny - 1);
-          if ((iterate = box_cg_cheaper(a, rmax, stop, i1 - i0 + 1, yhi - ylo + 1))) break;
+          if ((iterate = box_cg_ns(a, rmax, stop, i1 - i0 + 1, yhi - ylo + 1) < direct)) break;
         }
       }
     }
