@@ -482,8 +482,8 @@ constexpr float DCT_ERR = 1e-6f;
 // stopping rule's max(tol max theta_B, atol), at most maxit times or until the
 // residual stops falling (the rounding of eta itself).  solved:
 // whether the prediction was not just accepted.  Returns false if a grid
-// barrier gave up.
-template <int BS>
+// barrier gave up.  FLAT: for 2D meshes alone.
+template <int BS, bool FLAT = false>
 __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team& T, EtaOut& o, bool& solved) {
   const int nx = a.g.nx;
   const bool v4 = (nx & 3) == 0 && (a.g.pitch & 3) == 0 && al16(a.c) && al16(a.eta) && al16(a.r) && al16(a.p) &&
@@ -517,7 +517,7 @@ __device__ __forceinline__ bool eta_solve_team(const EtaArgs& a, DctSm& S, Team&
         const int mx = box_margin(a.cx, rmax, stop);
         i0 = max(32 * lo - mx, 0) & ~3;
         i1 = min((32 * hi + 31 + mx) | 3, nx - 1);  // whole quads where nx has them
-        const float direct = a.g.dim == 3 ? direct_ns(a, i1 - i0 + 1) : 0.0f;
+        const float direct = !FLAT && a.g.dim == 3 ? direct_ns(a, i1 - i0 + 1) : 0.0f;
         if (direct > CG_START_NS + CG_ITER_NS) {
           int ylo = a.g.ny, yhi = -1;
           for (int t = threadIdx.x & 31; t < a.tiles; t += 32)

@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(NTH, PLANE_MINB) step2d_kernel(const __grid_co
       if (blockIdx.x == 0 && tid < ETA_WORDS) eta_words(e.bar, ~step & 1)[tid] = 0u;
       EtaOut o;
       bool solved;
-      ok = eta_solve_team<NTH>(e, D, T, o, solved);
+      ok = eta_solve_team<NTH, true>(e, D, T, o, solved);
       if (ok && solved) {
         eta_note(e, o, ok);
         if (o.sync) ok = team_sync(e, T);
