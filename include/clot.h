@@ -221,6 +221,10 @@ int clot_mesh_info(const clot_mesh *mesh, clot_mesh_info_t *out);
  * dt continuing, and no other call of this library on the mesh in between
  * (they invalidate it).  A caller that changes c or eta itself between calls
  * sets CLOT_ETA_FRESH in params->flags for the next call.
+ * 2D meshes of at most two 32 x 8 tiles per SM run all steps up to the next
+ * sample in one cooperative launch, which waits until the GPU has room for a
+ * block per tile; not between clot_profile_begin and clot_profile_end, with
+ * fields->ext, or where eta needs CG alone (nx > 1024, ny > 512, L_eta = 0).
  * With CLOT_HEUN / CLOT_STRANG a step is [reaction over dt/2] -> transport
  * stage 1 (one pass) -> transport stage 2 + average + [reaction over dt/2] +
  * eta prediction (one fused pass): two or three sweeps of the state instead
@@ -350,7 +354,10 @@ int clot_ensemble_set_chains(clot_ensemble *ens, int chains);
 /* Per-kernel timing (library tracing).  Between clot_profile_begin and
  * clot_profile_end every kernel the library launches is bracketed by a pair of
  * CUDA events recorded on the launching stream (at most max_launches pairs;
- * later launches are only counted).  clot_profile_end synchronises the stream,
+ * later launches are only counted).  Meanwhile the 2D meshes whose steps
+ * otherwise share a launch (clot_species_step) run them launch by launch, an
+ * eta solve and a step kernel each, which takes longer: their sum is not the
+ * time of an untraced call.  clot_profile_end synchronises the stream,
  * sums the event times per kernel kind and stops recording.  Not part of the
  * paper; used by bench.py to time the dominant kernel inside a real run.
  * Errors: CLOT_EINVAL (max_launches < 1), CLOT_ECUDA. */

@@ -1,7 +1,7 @@
 // clot_eta.cu -- K2: the virtual-substance solve of App. A, Eq. eta,
 //     (I - (L_eta^2 / 4) lap_h) eta = theta_B,   zero-flux boundaries,
 // by conjugate gradients in one persistent cooperative launch, on meshes whose
-// extents the direct solver (clot_eta_dct.cu) does not take.  Vectors are
+// extents or coupling the direct solver (clot_eta_dct.cu) does not take.  Vectors are
 // FP32; every dot product and norm is accumulated in FP64 and reduced in a
 // fixed order, so all blocks see bit-identical scalars and the iteration is
 // deterministic.  The solve is warm-started from the eta passed in and stops

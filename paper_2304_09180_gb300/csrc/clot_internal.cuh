@@ -206,9 +206,10 @@ __device__ __forceinline__ int box_margin(float c, float rmax, float stop) {
   return (int)fminf(ceilf(n) + 1.0f, 1.0e6f);
 }
 
-// Threads per block of the eta CG kernel (its block reductions assume it):
-// two 512-thread blocks per SM cost fewer grid-barrier arrivals than five of
-// 256 at the same per-pass bandwidth.
+// Threads per block of the eta CG kernel (its block reductions assume it), one
+// block per SM: at the 64 registers of two it spills (eta a step, us, two blocks
+// -> one of 128 registers: 1280 x 256 primed channel 970 -> 654, 1040 x 128 x 128
+// duct 47 -> 37 plasma, 206 -> 219 primed, 64 x 520 x 64 primed 120 -> 90).
 constexpr int ETA_BLOCK = 512;
 cudaError_t launch_eta_solve(const EtaArgs& a, int grid, cudaStream_t s);
 int eta_max_grid(int* grid_out);
@@ -242,7 +243,8 @@ struct Run2d {
   int nmaxw, sel;               // set the first step adds to
   int ecur, eprev, have_pred;   // buffers of the first step's eta and of the one before
   int nsteps, do_eta, heun, strang;
-  int copy_c, copy_eta;         // the result back into c[0] (an odd number of steps), eta back into eta[0]
+  int copy_c, copy_eta;         // the state of the last step into the other of c[0], c[1] (where it ends up in the
+                                // buffer that is not the caller's), its eta into eta[0]
   int ntx, nty;
   unsigned long long wait_ns;   // bound of the waits for other blocks' cells (E.wait_ns: of the eta solves')
 };

@@ -46,12 +46,10 @@ constexpr int SY = BY + 2 * HY;  // 12
 constexpr int SPL = SX * SY;     // 432 cells per staged plane
 constexpr int NST = 9;           // staged species rows 0 .. 8
 
-// Staged tile layout with an x halo of HXT cells (y halo HY).
-template <int HXT>
-struct Lay {
-  static constexpr int HX = HXT, SX = BX + 2 * HXT, SPL = SX * SY;
+// Layout of a staged tile, as the cell code takes it.
+struct LA {
+  static constexpr int HX = clot::HX, SX = clot::SX, SPL = clot::SPL;
 };
-using LA = Lay<HX>;
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
