@@ -694,6 +694,7 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       if (!(p->flags & CLOT_NO_SIGMA) && (rc = sample_sigma(m, f, p, dt, s))) return rc;
       A.K.has_sigma = (!(p->flags & CLOT_NO_SIGMA) && f->n_samples > 0) ? 1 : 0;
       R.nsteps = 0;
+      const double t0 = f->t;
       do {
         ++R.nsteps;
         f->t += dt;
@@ -714,7 +715,9 @@ static int species_steps(clot_mesh* m, clot_fields* f, const clot_fluxes* fl, co
       const bool last = done == nsteps;
       R.copy_c = last && cur != f->c && !f->c_next;
       R.copy_eta = last && do_eta && (ep != 0 || ec == 0);
-      CUDA_OK(launch_steps_2d(R, s));
+      const cudaError_t launched = launch_steps_2d(R, s);
+      if (launched != cudaSuccess) f->t = t0;  // none of these steps was taken
+      CUDA_OK(launched);
       if (R.copy_c) cur = f->c;
       if (R.copy_eta) {
         if (ec == 0) ec = 3 - ep;
