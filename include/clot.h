@@ -367,7 +367,8 @@ typedef struct {
   int timed;                             /* launches with event pairs */
   int eta_iters;                         /* CG iterations or direct solves summed over the eta solves */
   int eta_accepted;                      /* eta solves that accepted the predicted eta */
-  int eta_box;                           /* eta solves that corrected the predicted eta on a box or slab (App. A, Eq. eta) */
+  int eta_box;                           /* eta solves that corrected the predicted eta on a box or slab (App. A,
+                                            Eq. eta) */
   int eta_box_fallback;                  /* box corrections that missed the stopping rule and continued on the mesh */
 } clot_profile_t;
 /* Not part of the paper (tracing): start recording; see above. */
